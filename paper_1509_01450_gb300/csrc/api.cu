@@ -84,7 +84,7 @@ static void free_plan(sg_plan* p)
     if (p->bstream) cudaStreamDestroy(p->bstream);
     // wc lies inside wb's allocation
     void* bufs[] = {p->tw, p->wa, p->wb, p->kr, p->kp, p->wpre, p->wpost, p->tw64, p->cells, p->keff,
-                    p->h_sigma, p->h_fr, p->h_fp, p->derr, p->egr, p->egp, p->wtab, p->wtmp, p->xf, p->xw,
+                    p->kfr, p->kfp, p->twx, p->h_sigma, p->h_fr, p->h_fp, p->derr, p->egr, p->egp, p->wtab, p->wtmp, p->xf, p->xw,
                     p->tcm};
     for (void* b : bufs)
         sg_free(b);
@@ -179,6 +179,10 @@ sg_status sg_plan_create(sg_plan** out, int nu, int nphi, double u_min, double d
         (st = dev_alloc(p, &p->wpost, nu * p->elem)) || (st = dev_alloc(p, (void**)&p->derr, 16)) ||
         (st = dev_alloc(p, (void**)&p->cells, (size_t)6 * (2 * nu + 1) * nphi * sizeof(double))) ||
         (st = dev_alloc(p, (void**)&p->keff, (size_t)2 * (2 * nu - 1) * nphi * sizeof(double))) ||
+        // the fixed-point passes' tables, where either direction has such transforms
+        (dtype != SG_F32 && (nphi >= 256 || nu >= 128) && (st = dev_alloc(p, &p->twx, fx_twiddle_bytes()))) ||
+        (dtype != SG_F32 && nu >= 128 &&
+         ((st = dev_alloc(p, &p->kfr, nk * 16)) || (st = dev_alloc(p, &p->kfp, nk * 16)))) ||
         (dtype == SG_F32X2 && ((st = dev_alloc(p, &p->xf, (size_t)3 * nu * nphi * sizeof(dfloat))) ||
                                (st = dev_alloc(p, &p->xw, (size_t)2 * nphi * sizeof(dfloat)))))) {
         free_plan(p);
@@ -207,6 +211,10 @@ sg_status sg_plan_create(sg_plan** out, int nu, int nphi, double u_min, double d
         t64[2 * j + 1] = im[j];
     }
     if (cudaMemcpy(p->tw64, t64.data(), SG_NMAX * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess) {
+        free_plan(p);
+        return SG_ERR_CUDA;
+    }
+    if (p->twx && cudaMemcpy(p->twx, fx_twiddles(), fx_twiddle_bytes(), cudaMemcpyHostToDevice) != cudaSuccess) {
         free_plan(p);
         return SG_ERR_CUDA;
     }
@@ -342,6 +350,7 @@ sg_status sg_plan_load(sg_plan** out, const char* path, cudaStream_t stream)
         cudaMemcpyAsync(p->kp, buf.data() + kb, kb, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
         cudaMemcpyAsync(p->wpre, buf.data() + 2 * kb, wb, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
         cudaMemcpyAsync(p->wpost, buf.data() + 2 * kb + wb, wb, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+        (p->kfr && launch_fx_spectra(view(p), p->dtype == SG_F32X2, stream) != cudaSuccess) ||
         cudaStreamSynchronize(stream) != cudaSuccess) {
         cudaGetLastError();
         sg_plan_destroy(p);
@@ -521,6 +530,7 @@ sg_status sg_kernels_build(sg_plan* p, const sg_build_opts* opts, cudaStream_t s
                         : p->dtype == SG_F32X2
                             ? launch_spectra<dfloat2>(v, nsr, nsp, W, (dfloat2*)p->kr, (dfloat2*)p->kp, stream)
                             : launch_spectra<double2>(v, nsr, nsp, W, (double2*)p->kr, (double2*)p->kp, stream);
+        if (e == cudaSuccess && p->kfr) e = launch_fx_spectra(v, p->dtype == SG_F32X2, stream);
         if (e != cudaSuccess) {
             ret = SG_ERR_CUDA;
             goto done;
@@ -559,9 +569,19 @@ static sg_status check_fields(const sg_plan* p, const void* a, const void* b, co
     return SG_OK;
 }
 
+// A compensated plan whose rows and columns both have fixed-point passes runs
+// them on its FP64 fields directly (1024 x 2048, forward and adjoint: 856 ->
+// 379 us).  The edge and wedge updates between the passes read double-float
+// spectra and tables, so plans with them keep the double-float passes.
+static bool fx_double_path(const sg_plan* p, const PlanView& v)
+{
+    return !p->edges && !p->wedge && fx_rows_ok(v) && fx_cols_ok(v);
+}
+
 // The passes on the plan's working type.  The compensated plans (SG_F32X2)
-// take and give FP64 fields: their inputs are split into double-float
-// working fields first and the results rounded back to FP64 after.
+// take and give FP64 fields; where they do not run on the fixed-point passes,
+// their inputs are split into double-float working fields first and the
+// results rounded back to FP64 after.
 static cudaError_t run_forward(sg_plan* p, PlanView v, const void* sigma, void* Fr, void* Fp, cudaStream_t st,
                                cudaEvent_t* ev = nullptr, bool direct = false)
 {
@@ -569,6 +589,10 @@ static cudaError_t run_forward(sg_plan* p, PlanView v, const void* sigma, void* 
         return launch_forward<float>(v, (const float*)sigma, (float*)Fr, (float*)Fp, st, ev, direct);
     if (p->dtype == SG_F64)
         return launch_forward<double>(v, (const double*)sigma, (double*)Fr, (double*)Fp, st, ev, direct);
+    if (fx_double_path(p, v)) {
+        v.wdf = 1;
+        return launch_forward<double>(v, (const double*)sigma, (double*)Fr, (double*)Fp, st, ev, direct);
+    }
     const size_t n = (size_t)p->nu * p->nphi;
     dfloat* const xs = (dfloat*)p->xf;
     dfloat* const xr = xs + n;
@@ -590,6 +614,10 @@ static cudaError_t run_backward(sg_plan* p, PlanView v, const void* gr, const vo
     if (p->dtype == SG_F32) return launch_backward<float>(v, (const float*)gr, (const float*)gp, (float*)gs, st, ev);
     if (p->dtype == SG_F64)
         return launch_backward<double>(v, (const double*)gr, (const double*)gp, (double*)gs, st, ev);
+    if (fx_double_path(p, v)) {
+        v.wdf = 1;
+        return launch_backward<double>(v, (const double*)gr, (const double*)gp, (double*)gs, st, ev);
+    }
     const size_t n = (size_t)p->nu * p->nphi;
     dfloat* const xr = (dfloat*)p->xf;
     dfloat* const xp = xr + n;

@@ -35,13 +35,10 @@
 // after P2 (inside P2 for FP32 with 16 points per thread) and its transpose
 // after P2b.  FP32 transforms of 2^8 .. 2^13 points run instances with the
 // length fixed at compile time, compiled in fftconv_lg<LG>.cu.
-#include <map>
 #include <mutex>
-#include <tuple>
-
-#include <nvtx3/nvToolsExt.h>
 
 #include "sg_internal.cuh"
+#include "sg_launch.cuh"
 
 namespace sg {
 
@@ -2037,98 +2034,6 @@ static Shape shape_for(int n, int min_threads)
     return s;
 }
 
-// Dynamic shared memory above the 48 KB default needs an opt-in; carveout
-// asks for the largest shared-memory split of L1 (several blocks of a
-// shared-memory-heavy kernel per SM).  Done once per kernel, device and
-// size: later launches (for example while a stream is being captured) make
-// no attribute calls.
-struct LaunchCache {
-    std::mutex mu;
-    std::map<std::tuple<const void*, int, int, size_t>, int> occ;  // (kernel, device, threads, smem) -> blocks/SM
-    std::map<std::tuple<const void*, int>, size_t> smem;            // (kernel, device) -> opted-in bytes
-};
-static LaunchCache& launch_cache()
-{
-    static LaunchCache c;
-    return c;
-}
-static int current_device()
-{
-    int d = 0;
-    if (cudaGetDevice(&d) != cudaSuccess) {
-        cudaGetLastError();
-        d = 0;
-    }
-    return d;
-}
-
-template <typename K>
-static cudaError_t set_smem(K kernel, size_t smem, bool carveout = false)
-{
-    LaunchCache& c = launch_cache();
-    const auto key = std::make_tuple((const void*)kernel, current_device());
-    std::lock_guard<std::mutex> lock(c.mu);
-    auto it = c.smem.find(key);
-    if (it != c.smem.end() && it->second >= smem) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && carveout)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e == cudaSuccess) c.smem[key] = it != c.smem.end() && it->second > smem ? it->second : smem;
-    return e;
-}
-
-// NVTX range around the enqueue of one pass (visible in Nsight timelines;
-// near-free when no tool is attached)
-struct PassRange {
-    explicit PassRange(const char* name) { nvtxRangePushA(name); }
-    ~PassRange() { nvtxRangePop(); }
-};
-
-// Launch with programmatic stream serialization: the kernel may start while
-// the previous one on the stream finishes; it waits (sg_grid_dep_wait)
-// before it reads that kernel's results.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
-                              Args&&... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
-// Blocks of a kernel resident on the GPU at once (occupancy x SMs), cached
-// per kernel, device and launch shape.
-template <typename K>
-static int resident_blocks(K kernel, int threads, size_t smem, int sms)
-{
-    LaunchCache& c = launch_cache();
-    const auto key = std::make_tuple((const void*)kernel, current_device(), threads, smem);
-    int occ = 0;
-    {
-        std::lock_guard<std::mutex> lock(c.mu);
-        auto it = c.occ.find(key);
-        if (it != c.occ.end()) occ = it->second;
-    }
-    if (occ == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem) != cudaSuccess || occ < 1) {
-            cudaGetLastError();
-            occ = 1;
-        }
-        std::lock_guard<std::mutex> lock(c.mu);
-        c.occ[key] = occ;
-    }
-    return occ * (sms > 0 ? sms : 1);
-}
-
 // Grid of a persistent row pass: as many blocks as fit on the GPU at once
 // (each loops over row blocks), at most one per row block.
 template <typename K>
@@ -2321,6 +2226,8 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
                                   (const float*)p.wpre, (float2*)p.wa, p.nu, (const float2*)p.tw, p.err, wave)) !=
                 cudaSuccess)
                 return err;
+        } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
+            if ((err = launch_fx_r2c(p, (const double*)sigma, nullptr, st)) != cudaSuccess) return err;
         } else {
             Shape s = shape_for<V>(p.nphi, sizeof(T) == 8 ? 64 : 256);
             const int R = 2 * s.slots, nblk = (p.nu + R - 1) / R;
@@ -2340,7 +2247,10 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
     }
     if (ev && (err = cudaEventRecord(ev[1], st)) != cudaSuccess) return err;
     bool edges_done = false;  // the column pass applied the edge-slope update itself
-    {
+    if (std::is_same<T, double>::value && fx_cols_ok(p)) {
+        PassRange range_("sg forward columns");
+        if ((err = launch_fx_cols(p, false, st)) != cudaSuccess) return err;
+    } else {
         PassRange range_("sg forward columns");
         const int L = 2 * p.nu, E = L >= 16 ? 16 : L;
         EdgeCoef<T> coef;
@@ -2384,6 +2294,8 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
                                   fr->c2r_smem, st, p.imaps[0], (const float*)p.wpost, (float*)Fr, (float*)Fp, p.nu,
                                   (const float2*)p.tw, p.err)) != cudaSuccess)
                 return err;
+        } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
+            if ((err = launch_fx_c2r(p, (double*)Fr, (double*)Fp, st)) != cudaSuccess) return err;
         } else {
             Shape s = shape_for<V>(p.nphi, sizeof(T) == 8 ? 64 : 256);
             const int R = 2 * s.slots, nblk = (p.nu + R - 1) / R;
@@ -2435,6 +2347,8 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
                                   (const float*)p.wpost, (float2*)p.wb, p.nu, (const float2*)p.tw, p.err, wave)) !=
                 cudaSuccess)
                 return err;
+        } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
+            if ((err = launch_fx_r2c(p, (const double*)gr, (const double*)gp, st)) != cudaSuccess) return err;
         } else {
             Shape s = shape_for<V>(p.nphi, row_min_threads(sizeof(T)));
             const int R = s.slots, nblk = (p.nu + R - 1) / R;
@@ -2453,7 +2367,10 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
         }
     }
     if (ev && (err = cudaEventRecord(ev[1], st)) != cudaSuccess) return err;
-    {
+    if (std::is_same<T, double>::value && fx_cols_ok(p)) {
+        PassRange range_("sg adjoint columns");
+        if ((err = launch_fx_cols(p, true, st)) != cudaSuccess) return err;
+    } else {
         PassRange range_("sg adjoint columns");
         const int L = 2 * p.nu, E = L >= 16 ? 16 : L;
         EdgeCoef<T> coef;
@@ -2493,6 +2410,8 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
                                   fr->c2r_smem, st, p.imaps[1], (const float*)p.wpre, (float*)gs, (float*)nullptr,
                                   p.nu, (const float2*)p.tw, p.err)) != cudaSuccess)
                 return err;
+        } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
+            if ((err = launch_fx_c2r(p, (double*)gs, nullptr, st)) != cudaSuccess) return err;
         } else {
             Shape s = shape_for<V>(p.nphi, sizeof(T) == 8 ? 64 : 256);
             const int R = 2 * s.slots, nblk = (p.nu + R - 1) / R;

@@ -1,0 +1,693 @@
+// fftfx.cuh -- the passes of the FP64 and compensated plans in 64-bit block
+// fixed point (sg_fx.cuh): FP64 fields and FP64 half spectra in memory, the
+// transforms and the products with the kernel spectra on the integer pipes.
+// Included by one translation unit per transform length (fftfx_lg<LG>.cu).
+//
+// The passes and their buffers are those of the run-time-length FP64 kernels
+// (fftconv.cu), element for element, so each may be replaced on its own and
+// the edge and wedge updates between them stay as they are.  A transform of N
+// points is held by N / 8 threads, 8 points each (32 registers); exchanges go
+// through 16-byte elements in shared memory, padded as sg_pad.  Each thread's
+// twiddles come from tables laid out by pass (fx_tw_base), read through L1:
+// their 61 bits would cost more to form by products.
+//
+// What bounds them: instruction issue, and before that the instruction cache.
+// A complex product is some 55 instructions, so unrolled passes are long: with
+// 16 points per thread, every pass unrolled and the inverse transforms apart
+// (140 KB of code in the column kernel) half of the cycles waited for
+// instructions.  Here the radix-8 passes of a kernel are one loop, and the
+// column kernels' three transforms share it (inverses as conj FFT conj).
+// Measured at 1024 x 2048, the FP64 pipe's kernels -> these, us: R2C rows 105
+// -> 32, columns 486 -> 111, C2R rows 195 -> 55; a forward call 781 -> 188.
+// Error of F_phi on a smooth disk of 256 x 512 against an 80-bit evaluation:
+// 1.6e-15 -> 1.6e-16 (F_r 4.4e-16 -> 2.2e-16).
+#pragma once
+#include "sg_internal.cuh"
+#include "sg_fx.cuh"
+
+namespace sg {
+
+template <int LG>
+struct FxShape {
+    static constexpr int N = 1 << LG, NT = N / 8;
+    static constexpr int SL = NT >= 128 ? 1 : 128 / NT;  // transforms per block: R2C rows, columns
+    static constexpr int RB = NT >= 64 ? 2 : 4;          // rows per block where 32-byte sectors need two
+    static constexpr size_t EX = (size_t)(N + N / 16 + 1) * sizeof(fx2);  // one exchange area
+    static constexpr size_t PARK = (size_t)N * sizeof(fx2);               // one parked spectrum
+};
+// blocks per SM the registers are bounded for: 768 threads' worth (80
+// registers); 512-thread blocks two (64 registers) where shared memory holds two
+constexpr int fx_minb(int threads, size_t smem) { return threads > 512 || 2 * smem > 220 * 1024 ? 1 : threads == 512 ? 2 : 768 / threads; }
+
+// OR / maximum over one transform's threads (whole warps) into a shared word, zero before
+__device__ __forceinline__ void fx_or_into(unsigned f, unsigned* word)
+{
+    f = __reduce_or_sync(0xffffffffu, f);
+    if ((threadIdx.x & 31) == 0) atomicOr(word, f);
+}
+__device__ __forceinline__ void fx_max_into(unsigned f, unsigned* word)
+{
+    f = __reduce_max_sync(0xffffffffu, f);
+    if ((threadIdx.x & 31) == 0) atomicMax(word, f);
+}
+
+__device__ __forceinline__ fx2 fx_ldg(const fx2* p)
+{
+    const longlong2 v = __ldg(reinterpret_cast<const longlong2*>(p));
+    return fx2{v.x, v.y};
+}
+__device__ __forceinline__ fxw fx_ldg(const fxw* p)
+{
+    const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+    return fxw{v.x, v.y, v.z, v.w};
+}
+
+// One transform of 2^LG points, thread t of 2^LG / 8 holding v[e] = x[t + e
+// NT] (components up to 2^59) on entry and X[t + e NT] (up to 2^62.5) on
+// return, natural order; the value is v 2^E throughout.  nrm: three zeroed
+// shared words of this transform.  sm is free on entry and on return.  Every
+// thread of the block calls.
+template <int LG, int DIR>
+__device__ __forceinline__ void fx_fft(fx2 (&v)[8], fx2* sm, unsigned* nrm, int t, const fxw* __restrict__ tw, int& E)
+{
+    constexpr int N = 1 << LG, NT = N / 8, R1 = 1 << fx_first_lg(LG), NP = fx_passes(LG);
+#pragma unroll
+    for (int s = 0; s < 8 / R1; s++) {
+        fx2 a[8];
+#pragma unroll
+        for (int r = 0; r < R1; r++) a[r] = v[s + r * (8 / R1)];
+        fx_dft<R1, DIR>(a);
+#pragma unroll
+        for (int r = 0; r < R1; r++) v[s + r * (8 / R1)] = a[r];
+    }
+    // butterfly t + s NT writes R1 neighbours
+#pragma unroll
+    for (int s = 0; s < 8 / R1; s++) {
+        fx2* q = sm + sg_pad((t + s * NT) * R1);
+#pragma unroll
+        for (int r = 0; r < R1; r++) q[r] = v[s + r * (8 / R1)];
+    }
+    int Ns = R1;  // length of the sub-transforms done so far
+    const fxw* w = tw + fx_tw_base(LG, 0);
+#pragma unroll 1
+    for (int p = 0; p < NP; p++) {
+        unsigned f = 0;
+#pragma unroll
+        for (int e = 0; e < 8; e++) f |= fx_fold(v[e]);
+        fx_or_into(f, nrm + p);
+        if (p > 0) {
+            const int Np = Ns >> 3, k = t & (Np - 1), base = (t - k) * 8 + k;
+#pragma unroll
+            for (int r = 0; r < 8; r++) sm[sg_pad(base + r * Np)] = v[r];
+        }
+        const int k = t & (Ns - 1);
+        __syncthreads();
+        const int s = max(fx_bits(nrm[p]) - FX_T, 0);
+#pragma unroll
+        for (int r = 0; r < 8; r++) v[r] = sm[sg_pad(t) + r * (NT + NT / 16)];
+        __syncthreads();
+        E += s;
+        const long long rnd = fx_round(s), h = s > 0 ? 1ll << (s - 1) : 0;
+        v[0] = fx2{(v[0].x + h) >> s, (v[0].y + h) >> s};
+#pragma unroll
+        for (int r = 1; r < 8; r++) {
+            v[r] = fx_cmul<DIR>(v[r], fx_ldg(w + (r - 1) * Ns + k), s, rnd);
+        }
+        fx_dft<8, DIR>(v);
+        w += 7 * Ns;
+        Ns <<= 3;
+    }
+}
+
+// a block's exponent from the largest high word; FX_BAD marks infinities and NaN
+__device__ __forceinline__ int fx_block_exp(unsigned abshi, int F) { return abshi >= 0x7ff00000u ? FX_BAD : fx_exp_of_field(F); }
+// conversions of a whole block: the exponent is the same for all, so the test is uniform
+__device__ __forceinline__ double2 fx_out(fx2 a, int E, bool safe)
+{
+    if (safe) return double2{fx_to_double(a.x, E), fx_to_double(a.y, E)};
+    return double2{fx_to_double_any(a.x, E), fx_to_double_any(a.y, E)};
+}
+__device__ __forceinline__ double fx_weight(const void* w, int i, int wdf)
+{
+    return wdf ? df_to_double(reinterpret_cast<const dfloat*>(w)[i]) : reinterpret_cast<const double*>(w)[i];
+}
+// whether a warp's rows are weighted (at p = 0 every weight is 1): an integer
+// comparison and a uniform branch around the products, which the FP64 pipe
+// would otherwise take 16 cycles a warp instruction for
+__device__ __forceinline__ bool fx_weighted(double w0, double w1)
+{
+    const long long one = 0x3ff0000000000000ll;
+    return __any_sync(0xffffffffu, __double_as_longlong(w0) != one || __double_as_longlong(w1) != one);
+}
+// 32 bytes (a whole L2 sector): two complex values of one mode
+__device__ __forceinline__ void fx_st256(double2* p, double2 a, double2 b, uint64_t pol)
+{
+    asm volatile("st.global.L2::cache_hint.v4.f64 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "d"(a.x), "d"(a.y), "d"(b.x),
+                 "d"(b.y), "l"(pol)
+                 : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// P1 / P1b: one complex transform of two real sequences per slot, split into
+// their half spectra.  Forward: rows 2p, 2p + 1 of sigma (x0), both halves to
+// A[m][2p], A[m][2p + 1] as one 32-byte store.  Adjoint: row i of gF_r (x0)
+// and gF_phi (x1), the halves to A and C, staged as S[m RB + row] and stored
+// by tensor copies of RB rows.
+// ---------------------------------------------------------------------------
+template <int LG, bool BWD>
+struct FxR2C {
+    typedef FxShape<LG> S;
+    static constexpr int SL = BWD ? S::RB : S::SL, THREADS = SL * S::NT;
+    static constexpr size_t SMEM = SL * S::EX + 128;
+    static constexpr int MINB = fx_minb(THREADS, SMEM);
+};
+template <int LG, bool BWD>
+__global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
+    k_fx_r2c(const double* __restrict__ x0, const double* __restrict__ x1, const void* __restrict__ wrow, int wdf,
+             double2* __restrict__ A, int nu, const fxw* __restrict__ tw, int* err,
+             const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapC)
+{
+    constexpr int N = 1 << LG, NT = N / 8, SL = FxR2C<LG, BWD>::SL;
+    extern __shared__ __align__(128) unsigned char smraw[];
+    __shared__ unsigned nrm[SL][5];
+    __shared__ double2 level[SL];
+    unsigned char* const area = smraw + ((128 - (sg_smem_u32(smraw) & 127)) & 127);
+    const int slot = threadIdx.x / NT, t = threadIdx.x % NT;
+    fx2* const sm = reinterpret_cast<fx2*>(area) + (size_t)slot * (N + N / 16 + 1);
+    if (t < 5) nrm[slot][t] = 0;
+    const int u = blockIdx.x * SL + slot, rows = BWD ? nu : nu / 2;
+    const bool live = u < rows;
+    const int i0 = BWD ? (live ? u : 0) : 2 * (live ? u : 0);
+    const double w0 = fx_weight(wrow, i0, wdf), w1 = BWD ? w0 : fx_weight(wrow, i0 + 1, wdf);
+    sg_grid_dep_launch();
+    sg_grid_dep_wait();  // the inputs may come from the previous kernel on the stream
+    const double* const r0 = x0 + (size_t)i0 * N + t;
+    const double* const r1 = BWD ? x1 + (size_t)i0 * N + t : r0 + N;
+    double2 z[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) z[e] = double2{r0[e * NT], r1[e * NT]};
+    if (fx_weighted(w0, w1)) {
+        asm volatile("" ::: "memory");  // stays a branch
+#pragma unroll
+        for (int e = 0; e < 8; e++) z[e] = double2{z[e].x * w0, z[e].y * w1};
+    }
+    unsigned h = 0;
+#pragma unroll
+    for (int e = 0; e < 8; e++) h = max(h, max(fx_abshi(z[e].x), fx_abshi(z[e].y)));
+    if (t == 0) level[slot] = z[0];
+    __syncthreads();
+    fx_max_into(h, &nrm[slot][3]);
+    __syncthreads();
+    h = nrm[slot][3];
+    const int F = fx_field(h);
+    int E = fx_block_exp(h, F);
+    // each row less its first value (exact in fixed point, and added to the
+    // DC mode below), at the exponent of what is left: a disk's axisymmetric
+    // part would otherwise set the exponent its other modes are rounded at
+    const fx2 c{fx_from_double(level[slot].x, F), fx_from_double(level[slot].y, F)};
+    fx2 v[8];
+    unsigned g = 0;
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        v[e] = fx2{fx_from_double(z[e].x, F) - c.x, fx_from_double(z[e].y, F) - c.y};
+        g |= fx_fold(v[e]);
+    }
+    fx_or_into(g, &nrm[slot][4]);
+    __syncthreads();
+    const int up = FX_T - fx_bits(nrm[slot][4]);
+#pragma unroll
+    for (int e = 0; e < 8; e++) v[e] = up >= 0 ? fx2{v[e].x << up, v[e].y << up} : fx2{v[e].x >> 1, v[e].y >> 1};
+    E -= max(up, -1);
+    fx_fft<LG, -1>(v, sm, nrm[slot], t, tw, E);
+    // X_a = (Z + conj Z[N - m]) / 2, X_b = (Z - conj Z[N - m]) / 2i
+#pragma unroll
+    for (int e = 0; e < 8; e++) sm[sg_pad(t + e * NT)] = v[e];
+    __syncthreads();
+    double2 xa[4], xb[4];
+    const bool safe = fx_exp_safe(E);
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+        const int m = t + e * NT;
+        const fx2 a{v[e].x >> 1, v[e].y >> 1};
+        fx2 b = sm[sg_pad((N - m) & (N - 1))];
+        b = fx2{b.x >> 1, b.y >> 1};
+        fx2 p{a.x + b.x, a.y - b.y}, q{a.y + b.y, b.x - a.x};
+        if (e == 0 && t == 0) {  // (DC, Nyquist) of both
+            const fx2 n = sm[sg_pad(N / 2)];
+            p = fx2{v[0].x, n.x};
+            q = fx2{v[0].y, n.y};
+        }
+        xa[e] = fx_out(p, E, safe);
+        xb[e] = fx_out(q, E, safe);
+        if (e == 0 && t == 0) {
+            xa[0].x += N * level[slot].x;
+            xb[0].x += N * level[slot].y;
+        }
+    }
+    const uint64_t keep = sg_policy_evict_last();  // the column pass reads the spectra from L2
+    if constexpr (!BWD) {
+        if (live) {
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const size_t at = (size_t)(t + e * NT) * nu + i0;
+                SG_IF_OK(sg_in((long long)at, 2, (long long)(N / 2) * nu), err, 901)
+                fx_st256(A + at, xa[e], xb[e], keep);
+            }
+        }
+    } else {
+        __syncthreads();  // the stages span the exchange areas
+        double2* const Sa = reinterpret_cast<double2*>(area);
+        double2* const Sc = Sa + (size_t)SL * (N / 2);
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            Sa[(t + e * NT) * SL + slot] = xa[e];
+            Sc[(t + e * NT) * SL + slot] = xb[e];
+        }
+        sg_fence_proxy_async();
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            const int ib = blockIdx.x * SL;
+            constexpr int MB = N / 2 < 256 ? N / 2 : 256, NBOX = N / 2 / MB;
+            for (int j = threadIdx.x; j < 2 * NBOX; j += 32) {
+                const double2* src = (j < NBOX ? Sa : Sc) + (size_t)(j % NBOX) * MB * SL;
+                SG_IF_OK(ib + SL <= nu && sg_smem_in(smraw, src, MB * SL * sizeof(double2)), err, 902)
+                sg_tma_store_2d(j < NBOX ? &mapA : &mapC, 2 * ib, (j % NBOX) * MB, src, keep);
+            }
+            sg_bulk_commit();
+            sg_bulk_wait_read();
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The products with the kernel spectra.  k1, k2: the two spectrum rows
+// (columns m > 0: Khat_r, Khat_phi of mode m; mode 0 packs DC and Nyquist:
+// Khat_r of both).  An entry's own exponent differs from its row's by dE
+// (0..63); the products wait unaligned until the block's largest is known,
+// and the entries' dE are then read again.
+// ---------------------------------------------------------------------------
+struct FxSpecRows {
+    const fx2 *k1, *k2;
+    bool z;  // mode 0
+};
+// kappa's entry for the frequency t + e NT, mirrored above N_u: Khat_r is
+// Hermitian, Khat_phi anti-Hermitian
+template <int NT>
+__device__ __forceinline__ int fx_spec_index(int t, int e) { return e < 4 ? t + e * NT : (8 - e) * NT - t; }
+template <int NT, bool SECOND>
+__device__ __forceinline__ fx2 fx_spec_at(const FxSpecRows& K, int t, int e, int& dE)
+{
+    fx2 w = fx_ldg((SECOND ? K.k2 : K.k1) + fx_spec_index<NT>(t, e));
+    dE = fx_spec_drop(w);
+    w = fx_spec_mant(w);
+    if (e > 4 || (e == 4 && t != 0)) {
+        if (SECOND && !K.z)
+            w.x = -w.x;
+        else
+            w.y = -w.y;
+    }
+    return w;
+}
+// the operand of the first (second) product at frequency k: the column's
+// spectrum, or for mode 0 the spectrum of its DC (Nyquist) part, from Z and
+// its mirror in sm
+template <int LG, bool SECOND>
+__device__ __forceinline__ fx2 fx_operand(fx2 a, const fx2* sm, int k, bool z)
+{
+    if (!z) return a;
+    const fx2 b = sm[sg_pad(((1 << LG) - k) & ((1 << LG) - 1))];
+    if (!SECOND) return fx2{(a.x >> 1) + (b.x >> 1), (a.y >> 1) - (b.y >> 1)};
+    return fx2{(a.y >> 1) + (b.y >> 1), (b.x >> 1) - (a.x >> 1)};
+}
+// DIR < 0: a K, DIR > 0: a conj K; at 2^-60 of the factors' scale
+template <int DIR>
+__device__ __forceinline__ fx2 fx_product(fx2 a, fx2 w, int dE, unsigned& top)
+{
+    const fx2 p = fx_cmul<DIR>(a, fx_digits(w.x, w.y), 0, fx_round(0));
+    top = max(top, (unsigned)(fx_bits(fx_fold(p)) + 64 - dE));
+    return p;
+}
+// a product at the block's exponent: shift = bits above FX_T of the largest
+template <int NT, bool SECOND>
+__device__ __forceinline__ fx2 fx_align(fx2 p, const FxSpecRows& K, int t, int e, int shift)
+{
+    const int2* w = reinterpret_cast<const int2*>((SECOND ? K.k2 : K.k1) + fx_spec_index<NT>(t, e));
+    const int d = ((__ldg(&w[0].x) & 7) | (__ldg(&w[1].x) & 7) << 3) + shift;
+    return fx2{fx_shift(p.x, d), fx_shift(p.y, d)};
+}
+
+template <int LG>
+struct FxCols {
+    typedef FxShape<LG> S;
+    static constexpr int THREADS = S::SL * S::NT;
+    static constexpr size_t SMEM = S::SL * (S::EX + S::PARK);
+    static constexpr int MINB = fx_minb(THREADS, SMEM);
+};
+
+// the N_u values of a column as the first half of a zero-padded transform;
+// top: a zeroed shared word.  Every thread of the block calls.
+template <int NT>
+__device__ __forceinline__ void fx_load_column(fx2 (&v)[8], const double2* __restrict__ in, unsigned* top, int& E)
+{
+    double2 a[4];
+    unsigned h = 0;
+#pragma unroll
+    for (int e = 0; e < 4; e++) a[e] = in[e * NT];
+#pragma unroll
+    for (int e = 0; e < 4; e++) h = max(h, max(fx_abshi(a[e].x), fx_abshi(a[e].y)));
+    fx_max_into(h, top);
+    __syncthreads();
+    h = *top;
+    const int F = fx_field(h);
+    E = fx_block_exp(h, F);
+#pragma unroll
+    for (int e = 0; e < 4; e++) v[e] = fx2{fx_from_double(a[e].x, F), fx_from_double(a[e].y, F)};
+#pragma unroll
+    for (int e = 4; e < 8; e++) v[e] = fx2{0, 0};
+}
+__device__ __forceinline__ fx2 fx_conj(fx2 a) { return fx2{a.x, -a.y}; }
+// a column's first N_u values, conjugated, to memory
+template <int NT>
+__device__ __forceinline__ void fx_store_column(const fx2 (&v)[8], double2* out, int E, bool live, long long at,
+                                                long long extent, int* err, int site)
+{
+    const bool safe = fx_exp_safe(E);
+    const uint64_t keep = sg_policy_evict_last();  // the row pass reads it from L2
+    if (live)
+#pragma unroll
+        for (int e = 0; e < 4; e++)
+            SG_IF_OK(sg_in(at + e * NT, 1, extent), err, site)
+            sg_st_hint(out + e * NT, fx_out(fx_conj(v[e]), E, safe), keep);
+}
+
+// P2: column m of A, zero-padded transform, times both spectra, two inverse
+// transforms cropped to N_u rows: B and C.
+template <int LG>
+__global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
+    k_fx_fwd_cols(const double2* __restrict__ A, const fx2* __restrict__ Kr, const fx2* __restrict__ Kp,
+                  double2* __restrict__ B, double2* __restrict__ C, int half, const fxw* __restrict__ tw, int* err)
+{
+    constexpr int L = 1 << LG, NT = L / 8, SL = FxShape<LG>::SL, nu = L / 2, KS = nu + 2;
+    extern __shared__ __align__(128) unsigned char smraw[];
+    __shared__ unsigned nrm[SL][12];  // three per transform, then the column's and the products' maxima
+    const int slot = threadIdx.x / NT, t = threadIdx.x % NT;
+    fx2* const sm = reinterpret_cast<fx2*>(smraw) + (size_t)slot * (L + L / 16 + 1);
+    fx2* const park = reinterpret_cast<fx2*>(smraw + SL * FxShape<LG>::EX) + (size_t)slot * L;
+    if (t < 12) nrm[slot][t] = 0;
+    const int m0 = blockIdx.x * SL + slot;
+    const bool live = m0 < half;
+    const int m = live ? m0 : half - 1;
+    const FxSpecRows K{Kr + (size_t)m * KS, m == 0 ? Kr + (size_t)half * KS : Kp + (size_t)m * KS, m == 0};
+    __syncthreads();
+    sg_grid_dep_launch();
+    sg_grid_dep_wait();  // A is the previous pass's result
+    fx2 v[8];
+    int E, E2 = 0, shift2 = 0;
+    fx_load_column<NT>(v, A + (size_t)m * nu + t, &nrm[slot][9], E);
+#pragma unroll 1
+    for (int pass = 0; pass < 3; pass++) {
+        fx_fft<LG, -1>(v, sm, &nrm[slot][3 * pass], t, tw, E);
+        if (pass > 0) {
+            fx_store_column<NT>(v, (pass == 1 ? B : C) + (size_t)m * nu + t, E, live, (long long)m * nu + t,
+                                (long long)half * nu, err, 903);
+            if (pass == 1) {
+#pragma unroll
+                for (int e = 0; e < 8; e++)
+                    v[e] = fx_conj(fx_align<NT, true>(park[t + e * NT], K, t, e, shift2));
+                E = E2;
+            }
+            continue;
+        }
+        if (blockIdx.x == 0) {  // holds mode 0: the mirror of every frequency
+#pragma unroll
+            for (int e = 0; e < 8; e++) sm[sg_pad(t + e * NT)] = v[e];
+            __syncthreads();
+        }
+        unsigned top1 = 0, top2 = 0;
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+            const int k = t + e * NT;
+            int d1, d2;
+            const fx2 w2 = fx_spec_at<NT, true>(K, t, e, d2);
+            park[k] = fx_product<-1>(fx_operand<LG, true>(v[e], sm, k, K.z), w2, d2, top2);
+            const fx2 w1 = fx_spec_at<NT, false>(K, t, e, d1);
+            v[e] = fx_product<-1>(fx_operand<LG, false>(v[e], sm, k, K.z), w1, d1, top1);
+        }
+        fx_max_into(top1, &nrm[slot][10]);
+        fx_max_into(top2, &nrm[slot][11]);
+        __syncthreads();
+        const int q1 = (int)nrm[slot][10] - 64, q2 = (int)nrm[slot][11] - 64;
+        const int EK1 = (int)fx_ldg(K.k1 + nu + 1).x, EK2 = (int)fx_ldg(K.k2 + nu + 1).x;
+        if (K.z) {  // Y_r = Y_DC + i Y_Nyquist at one exponent; the azimuthal force of both modes vanishes
+            const int EK = max(EK1, EK2), o1 = EK - EK1, o2 = EK - EK2, q = max(q1 - o1, q2 - o2) + 1;
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const fx2 a = fx_align<NT, false>(v[e], K, t, e, o1 + q - FX_T);
+                const fx2 b = fx_align<NT, true>(park[t + e * NT], K, t, e, o2 + q - FX_T);
+                v[e] = fx_conj(fx2{a.x - b.y, a.y + b.x});
+                park[t + e * NT] = fx2{0, 0};
+            }
+            E2 = E = E + EK + q + FX_WBITS - FX_T;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; e++) v[e] = fx_conj(fx_align<NT, false>(v[e], K, t, e, q1 - FX_T));
+            E2 = E + EK2 + q2 + FX_WBITS - FX_T;
+            shift2 = q2 - FX_T;
+            E = E + EK1 + q1 + FX_WBITS - FX_T;
+        }
+    }
+}
+
+// P2b: the columns of A and C, transforms, times conj Khat, summed, one
+// inverse transform cropped to N_u rows: B.  Mode 0 takes both its operands
+// (DC, Nyquist) from A: the azimuthal kernel vanishes there.
+template <int LG>
+__global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
+    k_fx_bwd_cols(const double2* __restrict__ A, const double2* __restrict__ C, const fx2* __restrict__ Kr,
+                  const fx2* __restrict__ Kp, double2* __restrict__ B, int half, const fxw* __restrict__ tw, int* err)
+{
+    constexpr int L = 1 << LG, NT = L / 8, SL = FxShape<LG>::SL, nu = L / 2, KS = nu + 2;
+    extern __shared__ __align__(128) unsigned char smraw[];
+    __shared__ unsigned nrm[SL][13];  // three per transform, the columns' maxima, the products' maxima
+    const int slot = threadIdx.x / NT, t = threadIdx.x % NT;
+    fx2* const sm = reinterpret_cast<fx2*>(smraw) + (size_t)slot * (L + L / 16 + 1);
+    fx2* const park = reinterpret_cast<fx2*>(smraw + SL * FxShape<LG>::EX) + (size_t)slot * L;
+    if (t < 13) nrm[slot][t] = 0;
+    const int m0 = blockIdx.x * SL + slot;
+    const bool live = m0 < half;
+    const int m = live ? m0 : half - 1;
+    const FxSpecRows K{Kr + (size_t)m * KS, m == 0 ? Kr + (size_t)half * KS : Kp + (size_t)m * KS, m == 0};
+    __syncthreads();
+    sg_grid_dep_launch();
+    sg_grid_dep_wait();  // A and C are the previous pass's results
+    fx2 v[8];
+    int E, Ep0 = 0;
+    fx_load_column<NT>(v, A + (size_t)m * nu + t, &nrm[slot][9], E);
+#pragma unroll 1
+    for (int pass = 0; pass < 3; pass++) {
+        fx_fft<LG, -1>(v, sm, &nrm[slot][3 * pass], t, tw, E);
+        if (pass == 2) {
+            fx_store_column<NT>(v, B + (size_t)m * nu + t, E, live, (long long)m * nu + t, (long long)half * nu, err,
+                                904);
+            break;
+        }
+        if (blockIdx.x == 0) {
+#pragma unroll
+            for (int e = 0; e < 8; e++) sm[sg_pad(t + e * NT)] = v[e];
+            __syncthreads();
+        }
+        unsigned top = 0;
+        if (pass == 0) {
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const int k = t + e * NT;
+                int d;
+                const fx2 w = fx_spec_at<NT, false>(K, t, e, d);
+                park[k] = fx_product<+1>(fx_operand<LG, false>(v[e], sm, k, K.z), w, d, top);
+            }
+            fx_max_into(top, &nrm[slot][11]);
+            Ep0 = E + (int)fx_ldg(K.k1 + nu + 1).x + FX_WBITS - FX_T;
+            __syncthreads();  // every mirror read is done
+            fx_load_column<NT>(v, (K.z ? A : C) + (size_t)m * nu + t, &nrm[slot][10], E);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                int d;
+                const fx2 w = fx_spec_at<NT, true>(K, t, e, d);
+                v[e] = fx_product<+1>(fx_operand<LG, true>(v[e], sm, t + e * NT, K.z), w, d, top);
+            }
+            fx_max_into(top, &nrm[slot][12]);
+            __syncthreads();  // every mirror read is done; the largest products are known
+            // both products at the larger one's exponent, one bit of room for their sum
+            const int q1 = (int)nrm[slot][11] - 64, q2 = (int)nrm[slot][12] - 64;
+            const int Ep1 = E + (int)fx_ldg(K.k2 + nu + 1).x + FX_WBITS - FX_T;
+            E = max(Ep0 + q1, Ep1 + q2) + 1;
+            const int s1 = E - Ep0 - FX_T, s2 = E - Ep1 - FX_T;
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const fx2 a = fx_align<NT, false>(park[t + e * NT], K, t, e, s1);
+                const fx2 b = fx_align<NT, true>(v[e], K, t, e, s2);
+                v[e] = fx_conj(K.z ? fx2{a.x - b.y, a.y + b.x} : fx_add(a, b));
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// P3 / P3b: RB rows per block.  Forward: per row Z = B + i C (Hermitian halves
+// expanded), inverse transform, F_r, F_phi = Re, Im.  Adjoint: per pair of
+// rows Z = S_i0 + i S_i1, gsigma of i0, i0 + 1 = Re, Im.  The rows' modes
+// arrive by 2-D tensor copies as S[m RB + r] (B, then C), each slot turns its
+// own modes into fixed point in place (once, not once per use), and the
+// exchange areas then lie over the stage.  The DC terms stay out of the
+// transform and are added to its rows: a disk's axisymmetric part would
+// otherwise set the exponent that its other modes are rounded at.
+// ---------------------------------------------------------------------------
+template <int LG, bool BWD>
+struct FxC2R {
+    typedef FxShape<LG> S;
+    static constexpr int SL = BWD ? S::RB / 2 : S::RB, THREADS = SL * S::NT;
+    static constexpr size_t STAGE = (size_t)S::RB * (S::N / 2) * sizeof(double2) * (BWD ? 1 : 2);
+    static constexpr size_t SMEM = (SL * S::EX > STAGE ? SL * S::EX : STAGE) + 128;
+    static constexpr int MINB = fx_minb(THREADS, SMEM);
+};
+template <int LG, bool BWD>
+__global__ void __launch_bounds__(FxC2R<LG, BWD>::THREADS, FxC2R<LG, BWD>::MINB)
+    k_fx_c2r(const void* __restrict__ wrow, int wdf, double* __restrict__ y0, double* __restrict__ y1, int nu,
+             const fxw* __restrict__ tw, int* err, const __grid_constant__ CUtensorMap mapB,
+             const __grid_constant__ CUtensorMap mapC)
+{
+    constexpr int N = 1 << LG, NT = N / 8, half = N / 2, RB = FxShape<LG>::RB, SL = FxC2R<LG, BWD>::SL;
+    const unsigned long long wlim = sg_wait_budget(err);  // read once, early
+    extern __shared__ __align__(128) unsigned char smraw[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ unsigned nrm[SL][4];
+    unsigned char* const area = smraw + ((128 - (sg_smem_u32(smraw) & 127)) & 127);
+    const int slot = threadIdx.x / NT, t = threadIdx.x % NT;
+    fx2* const sm = reinterpret_cast<fx2*>(area) + (size_t)slot * (N + N / 16 + 1);
+    if (t < 4) nrm[slot][t] = 0;
+    const int ib = blockIdx.x * RB, i0 = ib + (BWD ? 2 * slot : slot);
+    const double w0 = fx_weight(wrow, i0, wdf), w1 = BWD ? fx_weight(wrow, i0 + 1, wdf) : w0;
+    if (threadIdx.x == 0) sg_mbar_init(&bar, 1);
+    __syncthreads();
+    sg_grid_dep_launch();
+    sg_grid_dep_wait();  // the spectra are the previous pass's results
+    if (threadIdx.x < 32) {
+        constexpr int MB = half < 256 ? half : 256, NBOX = half / MB, NB = (BWD ? 1 : 2) * NBOX;
+        if (threadIdx.x == 0) sg_mbar_expect_tx(&bar, (uint32_t)(FxC2R<LG, BWD>::STAGE));
+        __syncwarp();
+        const uint64_t drop = sg_policy_evict_first();  // consumed here
+        for (int j = threadIdx.x; j < NB; j += 32) {
+            double2* dst = reinterpret_cast<double2*>(area) + (size_t)j * MB * RB;
+            SG_IF_OK(ib + RB <= nu && sg_smem_in(smraw, dst, MB * RB * sizeof(double2)), err, 905)
+            sg_tma_load_2d(dst, j < NBOX ? &mapB : &mapC, 2 * ib, (j % NBOX) * MB, &bar, drop);
+        }
+    }
+    if (__syncthreads_or(!sg_mbar_wait_bounded(&bar, 0, err, 1, wlim))) return;  // inputs never arrived
+    // this slot's two half spectra: element m at S0[m RB], S1[m RB]
+    double2* const S0 = reinterpret_cast<double2*>(area) + (BWD ? 2 * slot : slot);
+    double2* const S1 = BWD ? S0 + 1 : S0 + (size_t)half * RB;
+    const double dc0 = S0[0].x, dc1 = BWD ? S1[0].x : 0.0;  // (the azimuthal force has none)
+    int E;
+    {
+        double2 a[4], b[4];
+        unsigned h = 0;
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            a[e] = S0[(t + e * NT) * RB];
+            b[e] = S1[(t + e * NT) * RB];
+            if (e == 0 && t == 0) a[0].x = b[0].x = 0.0;
+            h = max(h, max(max(fx_abshi(a[e].x), fx_abshi(a[e].y)), max(fx_abshi(b[e].x), fx_abshi(b[e].y))));
+        }
+        fx_max_into(h, &nrm[slot][3]);
+        __syncthreads();
+        h = nrm[slot][3];
+        const int F = fx_field(h) + 1;  // one bit of room: Z adds two of them
+        E = fx_block_exp(h, F);
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            reinterpret_cast<fx2*>(S0)[(t + e * NT) * RB] = fx2{fx_from_double(a[e].x, F), fx_from_double(a[e].y, F)};
+            reinterpret_cast<fx2*>(S1)[(t + e * NT) * RB] = fx2{fx_from_double(b[e].x, F), fx_from_double(b[e].y, F)};
+        }
+    }
+    __syncthreads();
+    fx2 v[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        const int n = t + e * NT, mo = e < 4 ? n : (n == half ? 0 : N - n);
+        const fx2 a = reinterpret_cast<const fx2*>(S0)[mo * RB], b = reinterpret_cast<const fx2*>(S1)[mo * RB];
+        if (e == 0 && t == 0)
+            v[e] = fx2{0, 0};  // DC, added below
+        else if (e == 4 && t == 0)
+            v[e] = fx2{a.y, BWD ? b.y : 0};  // Nyquist
+        else if (e < 4)
+            v[e] = fx2{a.x - b.y, a.y + b.x};  // a + i b
+        else
+            v[e] = fx2{a.x + b.y, b.x - a.y};  // conj a + i conj b
+    }
+    __syncthreads();  // the exchange areas lie over the stage
+    fx_fft<LG, +1>(v, sm, nrm[slot], t, tw, E);
+    const bool safe = fx_exp_safe(E);
+    double* const o0 = y0 + (size_t)i0 * N + t;
+    double* const o1 = BWD ? y0 + (size_t)(i0 + 1) * N + t : y1 + (size_t)i0 * N + t;
+    double2 z[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        z[e] = fx_out(v[e], E, safe);
+        z[e].x += dc0;
+        if (BWD) z[e].y += dc1;
+    }
+    if (fx_weighted(w0, w1)) {
+        asm volatile("" ::: "memory");  // stays a branch
+#pragma unroll
+        for (int e = 0; e < 8; e++) z[e] = double2{z[e].x * w0, z[e].y * w1};
+    }
+    SG_IF_OK(i0 + (BWD ? 2 : 1) <= nu, err, 906)
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        o0[e * NT] = z[e].x;
+        o1[e * NT] = z[e].y;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// one length's kernels, reached through fx_kernels()
+// ---------------------------------------------------------------------------
+typedef void (*FxR2CFn)(const double*, const double*, const void*, int, double2*, int, const fxw*, int*, CUtensorMap,
+                        CUtensorMap);
+typedef void (*FxFwdColsFn)(const double2*, const fx2*, const fx2*, double2*, double2*, int, const fxw*, int*);
+typedef void (*FxBwdColsFn)(const double2*, const double2*, const fx2*, const fx2*, double2*, int, const fxw*, int*);
+typedef void (*FxC2RFn)(const void*, int, double*, double*, int, const fxw*, int*, CUtensorMap, CUtensorMap);
+struct FxKernels {
+    FxR2CFn r2c[2];  // forward, adjoint
+    FxC2RFn c2r[2];
+    FxFwdColsFn fwd_cols;
+    FxBwdColsFn bwd_cols;
+    int r2c_threads[2], c2r_threads[2], cols_threads;
+    size_t r2c_smem[2], c2r_smem[2], cols_smem;
+    int r2c_slots, cols_slots, rows;  // row pairs per forward R2C block, modes per column block, rows per other block
+};
+template <int LG>
+FxKernels make_fx_kernels()
+{
+    return FxKernels{{k_fx_r2c<LG, false>, k_fx_r2c<LG, true>},
+                     {k_fx_c2r<LG, false>, k_fx_c2r<LG, true>},
+                     k_fx_fwd_cols<LG>,
+                     k_fx_bwd_cols<LG>,
+                     {FxR2C<LG, false>::THREADS, FxR2C<LG, true>::THREADS},
+                     {FxC2R<LG, false>::THREADS, FxC2R<LG, true>::THREADS},
+                     FxCols<LG>::THREADS,
+                     {FxR2C<LG, false>::SMEM, FxR2C<LG, true>::SMEM},
+                     {FxC2R<LG, false>::SMEM, FxC2R<LG, true>::SMEM},
+                     FxCols<LG>::SMEM,
+                     FxShape<LG>::SL,
+                     FxShape<LG>::SL,
+                     FxShape<LG>::RB};
+}
+FxKernels fx_kernels_lg8();
+FxKernels fx_kernels_lg9();
+FxKernels fx_kernels_lg10();
+FxKernels fx_kernels_lg11();
+FxKernels fx_kernels_lg12();
+
+}  // namespace sg

@@ -31,6 +31,12 @@ struct sg_plan {
     void* wc;        // the fixed-length FP32 passes use as one buffer of (B, C) or (A, C) pairs
     void* kr;        // Khat_r, (nphi/2 + 1) x (nu + 2) complex
     void* kp;        // Khat_phi, same shape
+    // FP64 and compensated plans: the fixed-point passes' tables (sg_fx.cuh):
+    // both spectra as block fixed-point entries (null where 2 N_u has no
+    // fixed-point columns), the twiddles (null where neither direction has)
+    void* kfr;
+    void* kfp;
+    void* twx;
     void* wpre;      // beta^{p (i - i_ref)}, nu reals
     void* wpost;     // beta^{-p (i - i_ref)}
     int* derr;       // device: int flags of the passes' bounded waits, then (at +8 bytes)
@@ -90,6 +96,10 @@ struct PlanView {
     void *wa, *wb, *wc;
     const void* kr;
     const void* kp;
+    const void* kfr;        // fixed-point spectra and twiddles, or null
+    const void* kfp;
+    const void* twx;
+    int wdf;                // the row weights are double-floats (compensated plans on the FP64 path)
     const void* wpre;
     const void* wpost;
     int* err;
@@ -122,6 +132,10 @@ inline PlanView view(const sg_plan* p)
     v.wc = p->wc;
     v.kr = p->kr;
     v.kp = p->kp;
+    v.kfr = p->kfr;
+    v.kfp = p->kfp;
+    v.twx = p->twx;
+    v.wdf = 0;
     v.wpre = p->wpre;
     v.wpost = p->wpost;
     v.err = p->derr;
@@ -202,6 +216,21 @@ cudaError_t launch_dft_c2r(const PlanView& p, float* Fr, float* Fp, cudaStream_t
 cudaError_t launch_dft_r2c_adjoint(const PlanView& p, const float* gr, const float* gp, cudaStream_t st);
 cudaError_t launch_dft_c2r_adjoint(const PlanView& p, float* gs, cudaStream_t st);
 cudaError_t launch_dft_tc_batch(const TcArgs* d_args, int n, int dir, int max_nu, cudaStream_t st);
+// fftfx.cu: the passes in 64-bit block fixed point (sg_fx.cuh), over FP64
+// fields and FP64 half spectra.  *_ok: the plan's rows (N_phi of 256 .. 4096,
+// their tensor maps made) or columns (2 N_u of 256 .. 4096) run on them;
+// launch_fx_r2c's x1 and launch_fx_c2r's y1 are null for the forward R2C pass
+// and the adjoint C2R pass.
+bool fx_rows_ok(const PlanView& p);
+bool fx_cols_ok(const PlanView& p);
+cudaError_t launch_fx_r2c(const PlanView& p, const double* x0, const double* x1, cudaStream_t st);
+cudaError_t launch_fx_cols(const PlanView& p, bool adjoint, cudaStream_t st);
+cudaError_t launch_fx_c2r(const PlanView& p, double* y0, double* y1, cudaStream_t st);
+// the twiddle tables (host memory) and their size
+size_t fx_twiddle_bytes();
+const void* fx_twiddles();
+// p.kfr, p.kfp from p.kr, p.kp (df: stored as double-floats)
+cudaError_t launch_fx_spectra(const PlanView& p, bool df, cudaStream_t st);
 // every device allocation of the library, through the sg_test_fail_alloc
 // hook, and its release (sg_test_live_allocations counts the difference)
 cudaError_t sg_malloc(void** ptr, size_t bytes);
