@@ -41,6 +41,7 @@
 // MMAs and commits them to its "empty" mbarrier, and a buffer is refilled
 // only after that commit (every wait bounded).
 #include "sg_internal.cuh"
+#include "sg_launch.cuh"
 #include "sg_tc.cuh"
 
 #include <math.h>
@@ -173,6 +174,10 @@ __device__ __forceinline__ void dft_tc_tile(const TcArgs& a, int row_tile, int c
     __syncthreads();
     sg_tc_fence_after();
     const uint32_t tbase = tbase_s;
+    // the next pass may be placed from here on, not before: a later tensor-core
+    // pass's block that took this SM's tensor memory first would wait for this
+    // grid's end while this block waited for the tensor memory
+    sg_grid_dep_launch();
     const uint32_t idesc = sg_tc_idesc_tf32(TC_M, NT);
     const float wi = row_ok ? __ldg(&a.w[i]) : 0.f;
     // the CTA's column tile of the matrix stays resident: chunk c's two parts
@@ -200,7 +205,7 @@ __device__ __forceinline__ void dft_tc_tile(const TcArgs& a, int row_tile, int c
                                                                     c * TC_KC + h * (TC_KC / 2));
 #pragma unroll
                 for (int q = 0; q < QH; q++)
-                    v[g * QH + q] = row_ok ? __ldg(src + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[g * QH + q] = row_ok ? sg_ld_dep(src + q) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         } else {
             // modes c KC / 2 + h KC / 4 .. + KC / 4 - 1 of row i, two per float4
@@ -212,13 +217,13 @@ __device__ __forceinline__ void dft_tc_tile(const TcArgs& a, int row_tile, int c
                 if (row_ok) {
                     const size_t e0 = (size_t)(m0 + 2 * q) * nu + i, e1 = e0 + nu;
                     if constexpr (PAIRS && G == 2) {
-                        const float4 p0 = __ldg(a.pin + e0), p1 = __ldg(a.pin + e1);
+                        const float4 p0 = sg_ld_dep(a.pin + e0), p1 = sg_ld_dep(a.pin + e1);
                         v[q] = make_float4(p0.x, p0.y, p1.x, p1.y);
                         v[QH + q] = make_float4(p0.z, p0.w, p1.z, p1.w);
                     } else {
 #pragma unroll
                         for (int g = 0; g < G; g++) {
-                            const float2 b0 = __ldg(a.in[g] + e0), b1 = __ldg(a.in[g] + e1);
+                            const float2 b0 = sg_ld_dep(a.in[g] + e0), b1 = sg_ld_dep(a.in[g] + e1);
                             v[g * QH + q] = make_float4(b0.x, b0.y, b1.x, b1.y);
                         }
                     }
@@ -253,6 +258,7 @@ __device__ __forceinline__ void dft_tc_tile(const TcArgs& a, int row_tile, int c
         // three register sets in turn: the rows arrive two chunks after
         // their loads are issued, and no prefetched value is moved
         float4 va[G * QH], vb[G * QH], vc[G * QH];
+        sg_grid_dep_wait();  // the rows (or spectra) may come from the previous kernel on the stream
         load_rows(0, va);
         if (nch > 1) load_rows(1, vb);
         for (int c = 0; c < nch && !fail; c += 3) {
@@ -458,11 +464,10 @@ static cudaError_t tc_launch(const TcArgs& a, cudaStream_t st)
 {
     auto k = k_dft_tc<NT, DIR, G, PAIRS, NB>;
     const size_t smem = tc_smem_bytes<NT, G, NB>(a.N);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = set_smem(k, smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((a.nu + TC_M - 1) / TC_M, a.N / NT);
-    k<<<grid, TC_T, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k, grid, TC_T, smem, st, a);
 }
 
 // columns per CTA: 64 (32 for rows of 32); row buffers: three for one
@@ -499,14 +504,12 @@ cudaError_t launch_dft_tc_batch(const TcArgs* d_args, int n, int dir, int max_nu
     if (dir == 0) {
         auto k = k_dft_tc_batch<64, 0, 1, false, 3>;
         const size_t smem = tc_smem_bytes<64, 1, 3>(N);
-        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
+        if ((e = set_smem(k, smem)) != cudaSuccess) return e;
         k<<<grid, TC_T, smem, st>>>(d_args);
     } else {
         auto k = k_dft_tc_batch<64, 1, 2, true, 1>;
         const size_t smem = tc_smem_bytes<64, 2, 1>(N);
-        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
+        if ((e = set_smem(k, smem)) != cudaSuccess) return e;
         k<<<grid, TC_T, smem, st>>>(d_args);
     }
     return cudaGetLastError();

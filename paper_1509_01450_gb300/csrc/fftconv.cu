@@ -1657,10 +1657,15 @@ __global__ void __launch_bounds__(512) k_spec_cols(const double2* __restrict__ W
 #ifndef SG_ROWS_MINB
 #define SG_ROWS_MINB 3
 #endif
-template <int LG>
+// SMALL: blocks of one transform (two of 16 threads) instead of 256 threads'
+// worth, for grids whose rows would otherwise fill fewer blocks than the GPU
+// has SMs: a block's copy and barriers then cover only what it transforms.
+// Rows of 1024 points, 512 of them (32 / 64 blocks -> 128 / 256), us: R2C
+// 8.1 -> 5.6, C2R 7.7 -> 6.2.
+template <int LG, bool SMALL = false>
 struct RowUnit {
     static constexpr int N = 1 << LG, NT = N / 16;
-    static constexpr int GT = LG <= 12 ? 256 : 512;  // threads per block
+    static constexpr int GT = SMALL ? (NT < 32 ? 32 : NT) : LG <= 12 ? 256 : 512;  // threads per block
     static constexpr int TPG = GT / NT;              // paired transforms per block
     static constexpr int MINB = LG <= 12 ? SG_ROWS_MINB : 1;
     // the area: the transforms' exchange areas (C2 elements), plus the 1 KB alignment slack
@@ -1698,10 +1703,10 @@ __device__ __forceinline__ void split_real_pair2(const C2 (&w)[16], C2* sm, int 
     sync();  // every mirror read is done: the area is free
 }
 
-template <int LG>
+template <int LG, bool SMALL = false>
 __host__ __device__ __forceinline__ size_t rows_unit_smem_bytes()
 {
-    return RowUnit<LG>::SMEM;
+    return RowUnit<LG, SMALL>::SMEM;
 }
 
 // DIRECT (forward only): sigma is memory the GPU reaches only by plain loads
@@ -1715,14 +1720,14 @@ __host__ __device__ __forceinline__ size_t rows_unit_smem_bytes()
 // Returns false if the unit's inputs never arrived (the flag is set and the
 // unit's outputs are not written); the barrier's phase has then completed
 // only if its copies landed after all, which `landed` tells.
-template <int LG, bool BWD, bool DIRECT, bool PDL>
+template <int LG, bool BWD, bool DIRECT, bool PDL, bool SMALL = false>
 __device__ __forceinline__ bool rows_r2c_unit(const float* __restrict__ x0, const float* __restrict__ x1,
                                               const float* __restrict__ wrow, float2* __restrict__ out, int nu,
                                               const float2* __restrict__ tw, int* err, int u, int wave,
                                               unsigned char* smraw, uint64_t& bar, uint32_t phase,
                                               unsigned long long wlim, bool* landed = nullptr)
 {
-    typedef RowUnit<LG> RU;
+    typedef RowUnit<LG, SMALL> RU;
     constexpr int N = RU::N, NT = RU::NT, TPG = RU::TPG;
     constexpr int RPT = BWD ? 2 : 4;  // rows per transform
     constexpr int R = RPT * TPG;      // rows per block
@@ -1813,8 +1818,8 @@ __device__ __forceinline__ bool rows_r2c_unit(const float* __restrict__ x0, cons
     return true;
 }
 
-template <int LG, bool BWD, bool DIRECT = false>
-__global__ void __launch_bounds__(RowUnit<LG>::GT, RowUnit<LG>::MINB)
+template <int LG, bool BWD, bool DIRECT = false, bool SMALL = false>
+__global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MINB)
     k_rows_r2c(const float* __restrict__ x0, const float* __restrict__ x1, const float* __restrict__ wrow,
                float2* __restrict__ out, int nu, const float2* __restrict__ tw, int* err, int wave)
 {
@@ -1824,19 +1829,19 @@ __global__ void __launch_bounds__(RowUnit<LG>::GT, RowUnit<LG>::MINB)
     if (threadIdx.x == 0) sg_mbar_init(&bar, 1);
     __syncthreads();
     // the unit one wave later (wave = blocks resident at once) is prefetched
-    rows_r2c_unit<LG, BWD, DIRECT, true>(x0, x1, wrow, out, nu, tw, err, blockIdx.x, wave, smraw, bar, 0, wlim);
+    rows_r2c_unit<LG, BWD, DIRECT, true, SMALL>(x0, x1, wrow, out, nu, tw, err, blockIdx.x, wave, smraw, bar, 0, wlim);
 }
 
 // One unit of the row C2R pass (rows u R .. u R + R - 1), shared like
 // rows_r2c_unit; map: the tensor map in kernel-parameter or global memory.
-template <int LG, bool BWD, bool PDL>
+template <int LG, bool BWD, bool PDL, bool SMALL = false>
 __device__ __forceinline__ bool rows_c2r_unit(const CUtensorMap* map, const float* __restrict__ wrow,
                                               float* __restrict__ y0, float* __restrict__ y1, int nu,
                                               const float2* __restrict__ tw, int* err, int u, unsigned char* smraw,
                                               uint64_t& bar, uint32_t phase, unsigned long long wlim,
                                               bool* landed = nullptr)
 {
-    typedef RowUnit<LG> RU;
+    typedef RowUnit<LG, SMALL> RU;
     constexpr int N = RU::N, NT = RU::NT, TPG = RU::TPG, half = N / 2;
     constexpr int RPT = BWD ? 4 : 2;  // rows per transform
     constexpr int R = RPT * TPG;      // rows per block
@@ -1926,8 +1931,8 @@ __device__ __forceinline__ bool rows_c2r_unit(const CUtensorMap* map, const floa
 // map: 2-D tensor map over the input (forward: the pair layout, two 8-byte
 // units per row; adjoint: the single layout, one unit per row) with boxes
 // of 4 units x min(N/2, 256) modes and the 32-byte swizzle
-template <int LG, bool BWD>
-__global__ void __launch_bounds__(RowUnit<LG>::GT, RowUnit<LG>::MINB)
+template <int LG, bool BWD, bool SMALL = false>
+__global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MINB)
     k_rows_c2r(const __grid_constant__ CUtensorMap map, const float* __restrict__ wrow, float* __restrict__ y0,
                float* __restrict__ y1, int nu, const float2* __restrict__ tw, int* err)
 {
@@ -1936,7 +1941,7 @@ __global__ void __launch_bounds__(RowUnit<LG>::GT, RowUnit<LG>::MINB)
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) sg_mbar_init(&bar, 1);
     __syncthreads();
-    rows_c2r_unit<LG, BWD, true>(&map, wrow, y0, y1, nu, tw, err, blockIdx.x, smraw, bar, 0, wlim);
+    rows_c2r_unit<LG, BWD, true, SMALL>(&map, wrow, y0, y1, nu, tw, err, blockIdx.x, smraw, bar, 0, wlim);
 }
 
 // ===========================================================================
@@ -1960,40 +1965,51 @@ typedef void (*FwdColsFn)(const float2*, const float2*, const float2*, float2*, 
 typedef void (*BwdColsFn)(const float2*, const float2*, const float2*, const float2*, float2*, int, int, int,
                           const float2*, int*, const float*, const float*, const float*, EdgeCoef<float>);
 
-struct FixedPassKernels {
+struct FixedRowKernels {
     RowsR2CFn fwd_rows;         // k_rows_r2c, forward
     RowsR2CFn fwd_rows_direct;  // the same reading sigma from host memory the GPU can reach
     RowsR2CFn bwd_rows;         // k_rows_r2c, adjoint
-    RowsC2RFn fwd_rows_inv;  // k_rows_c2r, forward
-    RowsC2RFn bwd_rows_inv;  // k_rows_c2r, adjoint
-    size_t r2c_smem, c2r_smem;
+    RowsC2RFn fwd_rows_inv;     // k_rows_c2r, forward
+    RowsC2RFn bwd_rows_inv;     // k_rows_c2r, adjoint
+    size_t smem;
+    int threads;  // block size
+    int slots;    // paired transforms per block (RowUnit::TPG)
+};
+struct FixedPassKernels {
+    FixedRowKernels rows, small;  // blocks of 256 (512) threads, of one transform
     FwdColsFn fwd_cols;
     FwdColsFn fwd_cols_edge;        // with the edge-slope update
     FwdColsFn fwd_cols_edge_wedge;  // with the edge-slope and origin-wedge updates
     BwdColsFn bwd_cols;
     BwdColsFn bwd_cols_edge;  // with the transposed edge-slope update
-    int threads;  // block size of the row instances
-    int slots;    // paired transforms per row block (RowUnit::TPG)
+    // the row instances for passes of `rows_per_transform` rows each: the small
+    // blocks while the others are fewer than the SMs
+    const FixedRowKernels& pick(int nu, int rows_per_transform, int sms) const
+    {
+        return nu / (rows_per_transform * rows.slots) < sms ? small : rows;
+    }
 };
 
+template <int LG, bool SMALL>
+FixedRowKernels make_fixed_row_kernels()
+{
+    typedef RowUnit<LG, SMALL> RU;
+    return FixedRowKernels{k_rows_r2c<LG, false, false, SMALL>, k_rows_r2c<LG, false, true, SMALL>,
+                           k_rows_r2c<LG, true, false, SMALL>, k_rows_c2r<LG, false, SMALL>,
+                           k_rows_c2r<LG, true, SMALL>,        RU::SMEM,
+                           RU::GT,                             RU::TPG};
+}
 template <int LG>
 FixedPassKernels make_fixed_pass_kernels()
 {
     constexpr int NB = (1 << LG) / 16 > 256 ? 512 : 256;
-    return FixedPassKernels{k_rows_r2c<LG, false>,
-                            k_rows_r2c<LG, false, true>,
-                            k_rows_r2c<LG, true>,
-                            k_rows_c2r<LG, false>,
-                            k_rows_c2r<LG, true>,
-                            rows_unit_smem_bytes<LG>(),
-                            rows_unit_smem_bytes<LG>(),
+    return FixedPassKernels{make_fixed_row_kernels<LG, false>(),
+                            make_fixed_row_kernels<LG, (LG < 12)>(),  // one transform fills a block from 4096 points on
                             k_fwd_cols<float, 16, NB, LG>,
                             k_fwd_cols<float, 16, NB, LG, true>,
                             k_fwd_cols<float, 16, NB, LG, true, true>,
                             k_bwd_cols<float, 16, NB, LG>,
-                            k_bwd_cols<float, 16, NB, LG, true>,
-                            RowUnit<LG>::GT,
-                            RowUnit<LG>::TPG};
+                            k_bwd_cols<float, 16, NB, LG, true>};
 }
 
 // defined in fftconv_lg<LG>.cu
@@ -2061,6 +2077,18 @@ static int persistent_grid(K kernel, int threads, size_t smem, int nblk, int sms
 
 // threads a row-pass block should have at least (several slots per block)
 static int row_min_threads(size_t elem) { return elem == 4 ? 512 : 64; }
+// The block of an FP32 run-time row pass of `per` rows per slot: 256 threads'
+// worth of slots, halved down to a warp while the blocks are fewer than the
+// SMs.  64 rows of 64 points (one block -> four), us: R2C 6.8 -> 6.1, C2R 9.8 ->
+// 8.0.
+template <typename V>
+static Shape row_shape(int n, int nu, int per, int sms)
+{
+    int threads = sizeof(V) == 8 ? 256 : 64;
+    Shape s = shape_for<V>(n, threads);
+    while (sizeof(V) == 8 && threads > 32 && s.slots > 1 && nu < per * s.slots * sms) s = shape_for<V>(n, threads /= 2);
+    return s;
+}
 
 #ifndef SG_FFTCONV_DF  // the tensor maps are made once, in this translation unit
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -2179,15 +2207,19 @@ static cudaError_t launch_edges(const PlanView& p, bool adjoint, cudaStream_t st
 // The fixed-length instances of both transform lengths, when every pass of
 // the plan can run on them: FP32, N_phi and 2 N_u of 256 .. 8192 points, the
 // pair layout's tensor maps made, N_u a multiple of the row blocks.  The
-// passes then keep the column spectra in the pair layout.
+// passes then keep the column spectra in the pair layout.  Tensor-core rows
+// (short_dft) read and write that layout at any of their lengths, so with them
+// only the columns have to qualify (fr null where the rows have no instances):
+// a 4096 x 32 forward call, with the row passes chained by programmatic
+// launch as well, 29.2 -> 21.0 us.
 template <typename T>
 static bool fixed_path(const PlanView& p, const FixedPassKernels*& fr, const FixedPassKernels*& fc)
 {
     fr = fc = nullptr;
-    if (sizeof(T) != 4 || !p.imaps) return false;
+    if (sizeof(T) != 4) return false;
     const FixedPassKernels* a = fixed_pass_kernels(sg_ilog2(p.nphi));
     const FixedPassKernels* b = fixed_pass_kernels(sg_ilog2(2 * p.nu));
-    if (!a || !b || p.nu % (4 * a->slots) != 0) return false;
+    if (!b || (!p.tcm && (!p.imaps || !a || p.nu % (4 * a->rows.slots) != 0))) return false;
     fr = a;
     fc = b;
     return true;
@@ -2218,18 +2250,19 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
         if (sizeof(T) == 4 && p.tcm) {
             if ((err = launch_dft_r2c(p, (const float*)sigma, st)) != cudaSuccess) return err;
         } else if (p.pairs) {
-            const int nblk = p.nu / (4 * fr->slots);
-            auto k = sigma_direct ? fr->fwd_rows_direct : fr->fwd_rows;
-            if ((err = set_smem(k, fr->r2c_smem, true)) != cudaSuccess) return err;
-            const int wave = resident_blocks(k, fr->threads, fr->r2c_smem, p.sms);
-            if ((err = launch_pdl(k, nblk, fr->threads, fr->r2c_smem, st, (const float*)sigma, (const float*)nullptr,
+            const FixedRowKernels& rk = fr->pick(p.nu, 4, p.sms);
+            const int nblk = p.nu / (4 * rk.slots);
+            auto k = sigma_direct ? rk.fwd_rows_direct : rk.fwd_rows;
+            if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
+            const int wave = resident_blocks(k, rk.threads, rk.smem, p.sms);
+            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, (const float*)sigma, (const float*)nullptr,
                                   (const float*)p.wpre, (float2*)p.wa, p.nu, (const float2*)p.tw, p.err, wave)) !=
                 cudaSuccess)
                 return err;
         } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
             if ((err = launch_fx_r2c(p, (const double*)sigma, nullptr, st)) != cudaSuccess) return err;
         } else {
-            Shape s = shape_for<V>(p.nphi, sizeof(T) == 8 ? 64 : 256);
+            Shape s = row_shape<V>(p.nphi, p.nu, 2, p.sms);
             const int R = 2 * s.slots, nblk = (p.nu + R - 1) / R;
             const size_t smem = rows_fwd_smem_bytes<V>(p.nphi, s.slots);
             const CUtensorMap* mA = row_map(p, R, 0, p.nphi);
@@ -2287,17 +2320,17 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
         if (sizeof(T) == 4 && p.tcm) {
             if ((err = launch_dft_c2r(p, (float*)Fr, (float*)Fp, st)) != cudaSuccess) return err;
         } else if (p.pairs) {
-            const int nblk = p.nu / (2 * fr->slots);
-            auto k = fr->fwd_rows_inv;
-            if ((err = set_smem(k, fr->c2r_smem, true)) != cudaSuccess) return err;
-            if ((err = launch_pdl(k, nblk, fr->threads,
-                                  fr->c2r_smem, st, p.imaps[0], (const float*)p.wpost, (float*)Fr, (float*)Fp, p.nu,
+            const FixedRowKernels& rk = fr->pick(p.nu, 2, p.sms);
+            const int nblk = p.nu / (2 * rk.slots);
+            auto k = rk.fwd_rows_inv;
+            if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
+            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, p.imaps[0], (const float*)p.wpost, (float*)Fr, (float*)Fp, p.nu,
                                   (const float2*)p.tw, p.err)) != cudaSuccess)
                 return err;
         } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
             if ((err = launch_fx_c2r(p, (double*)Fr, (double*)Fp, st)) != cudaSuccess) return err;
         } else {
-            Shape s = shape_for<V>(p.nphi, sizeof(T) == 8 ? 64 : 256);
+            Shape s = row_shape<V>(p.nphi, p.nu, 2, p.sms);
             const int R = 2 * s.slots, nblk = (p.nu + R - 1) / R;
             const size_t smem = rows_inv_smem_bytes<V>(p.nphi, s.slots);
             const CUtensorMap* mB = row_map(p, R, 1, p.nphi);
@@ -2339,11 +2372,12 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
         if (sizeof(T) == 4 && p.tcm) {
             if ((err = launch_dft_r2c_adjoint(p, (const float*)gr, (const float*)gp, st)) != cudaSuccess) return err;
         } else if (p.pairs) {  // (A, C) pairs into wb
-            const int nblk = p.nu / (2 * fr->slots);
-            auto k = fr->bwd_rows;
-            if ((err = set_smem(k, fr->r2c_smem, true)) != cudaSuccess) return err;
-            const int wave = resident_blocks(k, fr->threads, fr->r2c_smem, p.sms);
-            if ((err = launch_pdl(k, nblk, fr->threads, fr->r2c_smem, st, (const float*)gr, (const float*)gp,
+            const FixedRowKernels& rk = fr->pick(p.nu, 2, p.sms);
+            const int nblk = p.nu / (2 * rk.slots);
+            auto k = rk.bwd_rows;
+            if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
+            const int wave = resident_blocks(k, rk.threads, rk.smem, p.sms);
+            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, (const float*)gr, (const float*)gp,
                                   (const float*)p.wpost, (float2*)p.wb, p.nu, (const float2*)p.tw, p.err, wave)) !=
                 cudaSuccess)
                 return err;
@@ -2403,17 +2437,17 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
         if (sizeof(T) == 4 && p.tcm) {
             if ((err = launch_dft_c2r_adjoint(p, (float*)gs, st)) != cudaSuccess) return err;
         } else if (p.pairs) {  // B from wa
-            const int nblk = p.nu / (4 * fr->slots);
-            auto k = fr->bwd_rows_inv;
-            if ((err = set_smem(k, fr->c2r_smem, true)) != cudaSuccess) return err;
-            if ((err = launch_pdl(k, nblk, fr->threads,
-                                  fr->c2r_smem, st, p.imaps[1], (const float*)p.wpre, (float*)gs, (float*)nullptr,
+            const FixedRowKernels& rk = fr->pick(p.nu, 4, p.sms);
+            const int nblk = p.nu / (4 * rk.slots);
+            auto k = rk.bwd_rows_inv;
+            if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
+            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, p.imaps[1], (const float*)p.wpre, (float*)gs, (float*)nullptr,
                                   p.nu, (const float2*)p.tw, p.err)) != cudaSuccess)
                 return err;
         } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
             if ((err = launch_fx_c2r(p, (double*)gs, nullptr, st)) != cudaSuccess) return err;
         } else {
-            Shape s = shape_for<V>(p.nphi, sizeof(T) == 8 ? 64 : 256);
+            Shape s = row_shape<V>(p.nphi, p.nu, 2, p.sms);
             const int R = 2 * s.slots, nblk = (p.nu + R - 1) / R;
             const size_t smem = rows_bwd_inv_smem_bytes<V>(p.nphi, s.slots);
             const CUtensorMap* mB = row_map(p, R, 1, p.nphi);

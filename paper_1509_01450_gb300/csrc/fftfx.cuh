@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
     const double* const r1 = BWD ? x1 + (size_t)i0 * N + t : r0 + N;
     double2 z[8];
 #pragma unroll
-    for (int e = 0; e < 8; e++) z[e] = double2{r0[e * NT], r1[e * NT]};
+    for (int e = 0; e < 8; e++) z[e] = double2{sg_ld_dep(r0 + e * NT), sg_ld_dep(r1 + e * NT)};
     if (fx_weighted(w0, w1)) {
         asm volatile("" ::: "memory");  // stays a branch
 #pragma unroll
@@ -352,7 +352,7 @@ __device__ __forceinline__ void fx_load_column(fx2 (&v)[8], const double2* __res
     double2 a[4];
     unsigned h = 0;
 #pragma unroll
-    for (int e = 0; e < 4; e++) a[e] = in[e * NT];
+    for (int e = 0; e < 4; e++) a[e] = sg_ld_dep(in + e * NT);
 #pragma unroll
     for (int e = 0; e < 4; e++) h = max(h, max(fx_abshi(a[e].x), fx_abshi(a[e].y)));
     fx_max_into(h, top);

@@ -540,6 +540,38 @@ __device__ __forceinline__ void sg_fence_proxy_async() { asm volatile("fence.pro
 __device__ __forceinline__ void sg_grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void sg_grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Loads of what a previous kernel wrote, after sg_grid_dep_wait: volatile, so
+// that they stay behind it.  (A load through a const __restrict__ pointer or
+// __ldg is free to move above the wait: the compiler takes its memory for
+// constant over the whole kernel.)
+__device__ __forceinline__ float2 sg_ld_dep(const float2* p)
+{
+    float2 r;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "l"(p) : "memory");
+    return r;
+}
+__device__ __forceinline__ float4 sg_ld_dep(const float4* p)
+{
+    float4 r;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
+                 : "l"(p)
+                 : "memory");
+    return r;
+}
+__device__ __forceinline__ double sg_ld_dep(const double* p)
+{
+    double r;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(r) : "l"(p) : "memory");
+    return r;
+}
+__device__ __forceinline__ double2 sg_ld_dep(const double2* p)
+{
+    double2 r;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(r.x), "=d"(r.y) : "l"(p) : "memory");
+    return r;
+}
+
 // ---------------------------------------------------------------------------
 // L2 eviction priorities.  The half-spectrum intermediates are written by one
 // pass and read, transposed, by the next; they are kept in L2 (evict_last)
