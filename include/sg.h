@@ -357,7 +357,7 @@ sg_status sg_forces_batched(const sg_batch_item* items, int n, cudaStream_t stre
  * stream) so that later sg_forces_batched calls with the same items, also
  * captured ones, take it.  Allocates the list's device memory, held until
  * one of the plans is destroyed: each item's own intermediate spectra (12
- * bytes per cell; items may share a plan), a descriptor of 256 bytes per
+ * bytes per cell; items may share a plan), a descriptor of 384 bytes per
  * item and 8 bytes per work item.  The library keeps the 4 lists prepared
  * last (a call with a new list of items builds one: host work and a
  * synchronising copy).  SG_ERR_UNSUPPORTED if the items do not qualify

@@ -27,7 +27,7 @@ namespace sg {
 
 // One disk, as the kernel sees it (aligned as its tensor map requires).
 struct BatchDisk {
-    CUtensorMap map;  // the plan's map over the pair layout (the C2R pass's input)
+    CUtensorMap maps[2];  // over the pairs P and the half spectra A (the column pass's copies)
     const float* sigma;
     float* Fr;
     float* Fp;
@@ -41,6 +41,7 @@ struct BatchDisk {
     int* err;
     int nu, nphi, lgr, lgc;  // sizes; log2 N_phi and log2 2 N_u
     int n_rows, n_cols, n_inv;  // items of the R2C, column and C2R passes
+    int rows_layout;            // 0: columns contiguous (tensor-core rows), 1: the row layout
     int rows_mult, cols_mult;   // units per row item (both row passes), mode groups per column item (tuned)
 };
 
@@ -70,7 +71,7 @@ __device__ __forceinline__ bool batch_inv(const BatchDisk& D, int u, unsigned ch
                                           uint32_t& ph, unsigned long long wlim)
 {
     bool landed = true;
-    rows_c2r_unit<LG, false, false>(&D.map, D.wpost, D.Fr, D.Fp, D.nu, D.tw, D.err, u, smraw, bar, ph, wlim, &landed);
+    rows_c2r_unit<LG, false, false>(reinterpret_cast<const float4*>(D.P), D.wpost, D.Fr, D.Fp, D.nu, D.tw, D.err, u, smraw, bar, ph, wlim, &landed);
     landed = __syncthreads_or(landed);
     if (landed) ph ^= 1;
     return landed;
@@ -108,7 +109,10 @@ __device__ __forceinline__ bool batch_cols(const BatchDisk& D, int g, unsigned c
                                  drop);
             }
             SG_IF_OK(sg_in((long long)ms * nu, nu, (long long)half * nu) && sg_smem_in(smraw, cs, ab), D.err, 802)
-            sg_bulk_g2s_hint(cs, D.A + (size_t)ms * nu, ab, &bar[0], drop);
+            if (D.rows_layout)
+                spec_load_column(cs, &D.maps[1], ms, nu / 4, &bar[0], drop);
+            else
+                sg_bulk_g2s_hint(cs, D.A + (size_t)ms * nu, ab, &bar[0], drop);
         }
     }
     const Twd<16, float2> twd = make_twd<16>(LGC, t, D.tw);
@@ -131,7 +135,24 @@ __device__ __forceinline__ bool batch_cols(const BatchDisk& D, int g, unsigned c
         if (fwd_cols_math<LGC, true>(v, sm, kr_s, kp_s, reinterpret_cast<C2*>(base), m, t, nu, LGC, twd, wait_spectra,
                                      w)) {
             const uint64_t keep = sg_policy_evict_last();  // the C2R pass reads the pairs from L2
+            if (D.rows_layout) {  // as k_fwd_cols: staged over the exchange area, then scattered
+                float4* const S = reinterpret_cast<float4*>(base);
+                const int sw = spec_swap(m);
+#pragma unroll
+                for (int e = 0; e < 8; e++)
+                    S[(t + e * NT) ^ sw] = make_float4(f2_lo(w[e].x), f2_lo(w[e].y), f2_hi(w[e].x), f2_hi(w[e].y));
+                sg_fence_proxy_async();
+            }
+            __syncthreads();
             float4* const P = reinterpret_cast<float4*>(D.P) + (size_t)m * nu;
+            if (D.rows_layout) {
+                if (t == 0) {
+                    SG_IF_OK(m < half && sg_smem_in(smraw, base, (uint32_t)nu * 16), D.err, 804)
+                    spec_store_column(&D.maps[0], m, nu / 2, base, keep);
+                    sg_bulk_commit();
+                    sg_bulk_wait_read();
+                }
+            } else
 #pragma unroll
             for (int e = 0; e < 8; e++)  // crop to N_u rows
                 SG_IF_OK(sg_in((long long)m * nu + t + e * NT, 1, (long long)half * nu), D.err, 803)
@@ -401,12 +422,11 @@ static sg_status make_list(const sg_batch_item* items, int n, const BatchTuning&
         memset(&d, 0, sizeof(d));
         d.A = (float2*)(b.d_work + off_a[i]);
         d.P = (float2*)(b.d_work + off_p[i]);
-        CUtensorMap maps[2];
-        if (!make_pair_maps(p->nu, p->nphi, d.A, d.P, maps)) {
+        if (!make_pair_maps(p->nu, p->nphi, d.A, d.P, d.maps)) {
             free_list(b);
             return SG_ERR_CUDA;
         }
-        d.map = maps[0];
+        d.rows_layout = p->short_dft ? 0 : 1;
         d.sigma = (const float*)items[i].sigma;
         d.Fr = (float*)items[i].F_r;
         d.Fp = (float*)items[i].F_phi;

@@ -22,7 +22,8 @@
 //
 // Half spectra along phi keep modes 0..N_phi/2-1, with the real DC and
 // Nyquist values packed into mode 0 as (DC, Nyquist).  A, B and C are all
-// mode-major, X[m N_u + i]: a column pass reads and writes whole contiguous
+// mode-major, X[m N_u + i] (the fixed-length FP32 passes use the row layout
+// below instead): a column pass reads and writes whole contiguous
 // columns, and the row passes move them through shared memory in 16-byte
 // units (stage_load / stage_store).
 //
@@ -423,6 +424,40 @@ __global__ void __launch_bounds__(NTB, (sizeof(T) == 4 && NTB == 256) ? 2 : 1) k
 }
 
 // ===========================================================================
+// The row layout of the fixed-length FP32 passes: half spectra in units of 32
+// bytes, one mode of four rows (single values) or of two rows (pairs {X, Y}),
+// unit (g, m) at g N_phi / 2 + m for row group g.  A row pass then reads or
+// writes whole contiguous rows of units (one bulk copy in, coalesced 32-byte
+// stores out); the transposition is the column pass's, whose tensor copies
+// gather or scatter a column's units (boxes of one mode x up to 256 groups)
+// while its other blocks compute.  In the layout's predecessor, columns
+// contiguous, the row passes' own copies took 0.64 box rows a clock and SM,
+// half of the C2R pass's time.  N_u x N_phi = 2048 x 4096, columns -> rows
+// contiguous, us: R2C 21.3 -> 18.4, columns 51.1 -> 51.2, C2R 31.5 -> 27.9;
+// adjoint 34.7 -> 29.3, 53.7 -> 57.0, 20.0 -> 18.3.
+// The unit's halves are swapped for modes with bit 2 set where the C2R pass
+// reads them (its 16-byte reads of neighbouring modes' units then meet no
+// bank twice).
+// ===========================================================================
+__host__ __device__ __forceinline__ int spec_box_rows(int groups) { return groups < 256 ? groups : 256; }
+// a column's units into (from) shared memory in row order, one thread; the
+// caller sets the barrier's expected bytes (commits the stores)
+__device__ __forceinline__ void spec_load_column(void* dst, const CUtensorMap* map, int m, int groups, uint64_t* bar,
+                                                 uint64_t policy)
+{
+    const int box = spec_box_rows(groups);
+    for (int g = 0; g < groups; g += box)
+        sg_tma_load_3d(static_cast<unsigned char*>(dst) + (size_t)g * 32, map, 0, m, g, bar, policy);
+}
+__device__ __forceinline__ void spec_store_column(const CUtensorMap* map, int m, int groups, const void* src,
+                                                  uint64_t policy)
+{
+    const int box = spec_box_rows(groups);
+    for (int g = 0; g < groups; g += box)
+        sg_tma_store_3d(map, 0, m, g, static_cast<const unsigned char*>(src) + (size_t)g * 32, policy);
+}
+
+// ===========================================================================
 // Forward P2: one phi-mode column m per block.  Shared memory: the FFT
 // exchange buffer (its first N_u entries double as the landing area of the
 // column), then Khat_r[m] and Khat_phi[m] (for m = 0: Khat_r of modes 0 and
@@ -476,10 +511,11 @@ __host__ __device__ __forceinline__ size_t cols_smem_bytes(int nu)
 // column pass runs one mode per block; the batched kernel (SLOTTED) runs
 // several modes of one disk side by side in a block, each on its own
 // shared memory, with every barrier taken by the whole block.
-template <int LG, bool SLOTTED, typename WaitFn>
+template <int LG, bool SLOTTED, typename WaitFn, typename Sync = SgSyncBlock>
 __device__ __forceinline__ bool fwd_cols_math(float2 (&v)[16], float2* sm, const float2* kr_s, const float2* kp_s,
                                               C2* xarea, int m, int t, int nu, int log2L,
-                                              const Twd<16, float2>& twd, WaitFn wait_spectra, C2 (&w)[16])
+                                              const Twd<16, float2>& twd, WaitFn wait_spectra, C2 (&w)[16],
+                                              const Sync& isync = Sync())
 {
     typedef float2 V;
     typedef float T;
@@ -519,7 +555,7 @@ __device__ __forceinline__ bool fwd_cols_math(float2 (&v)[16], float2* sm, const
         }
     }
     // both inverse transforms; their first exchange waits for every spectrum read
-    sg_fft_pair<+1, LG>(w, xarea, L, log2L, t, twd.h);
+    sg_fft_pair<+1, LG>(w, xarea, L, log2L, t, twd.h, isync);
     return true;
 }
 
@@ -531,7 +567,9 @@ __global__ void SG_FCOLS_BOUNDS(T, NTB, LG, EDGE) k_fwd_cols(const typename CX<T
                                                   typename CX<T>::t* __restrict__ Cp, int nu, int nphi, int log2L,
                                                   const typename CX<T>::t* __restrict__ tw, int* err,
                                                   const T* __restrict__ egr, const T* __restrict__ egp,
-                                                  const T* __restrict__ wpre, EdgeCoef<T> ecoef, WedgeArgs<T> wdg)
+                                                  const T* __restrict__ wpre, EdgeCoef<T> ecoef, WedgeArgs<T> wdg,
+                                                  const __grid_constant__ CUtensorMap mapA,
+                                                  const __grid_constant__ CUtensorMap mapP, int rows_layout)
 {
     const unsigned long long wlim = sg_wait_budget(err);  // read once, early
     if constexpr (LG > 0) {  // the length is a compile-time constant
@@ -580,8 +618,12 @@ __global__ void SG_FCOLS_BOUNDS(T, NTB, LG, EDGE) k_fwd_cols(const typename CX<T
     sg_grid_dep_wait();  // A is the previous pass's result
     if (t == 0) {
         sg_mbar_expect_tx(&bar[0], ab);
-        SG_IF_OK(sg_in((long long)m * nu, nu, (long long)half * nu) && sg_smem_in(smraw, sm, ab), err, 303)
-        sg_bulk_g2s_hint(sm, A + (size_t)m * nu, ab, &bar[0], drop);
+        SG_IF_OK(sg_in((long long)m * nu, nu, (long long)half * nu) && sg_smem_in(smraw, sm, ab), err, 303) {
+            if (LG > 0 && rows_layout)
+                spec_load_column(sm, &mapA, m, nu / 4, &bar[0], drop);
+            else
+                sg_bulk_g2s_hint(sm, A + (size_t)m * nu, ab, &bar[0], drop);
+        }
     }
     const Twd<E, V> twd = make_twd<E>(log2L, t, tw);
     const uint64_t keep = sg_policy_evict_last();  // the row pass reads B and C from L2
@@ -663,7 +705,33 @@ __global__ void SG_FCOLS_BOUNDS(T, NTB, LG, EDGE) k_fwd_cols(const typename CX<T
                 w[e] = C2{w[e].x + f2(wi * dr.x, wi * dq.x), w[e].y + f2(wi * dr.y, wi * dq.y)};
             }
         }
-        if constexpr (LG > 0) {
+        if (LG > 12 && rows_layout) {
+            // one block per SM: no other block computes while staged copies
+            // leave, so each thread stores its own
+            float4* const P = reinterpret_cast<float4*>(Br);
+            const int sw = spec_swap(m);
+#pragma unroll
+            for (int e = 0; e < E / 2; e++) {  // crop to N_u rows
+                const size_t at = spec_at(m, (t + e * NT) ^ sw, half, 1);
+                SG_IF_OK(sg_in((long long)at, 1, (long long)half * nu), err, 309)
+                sg_st_hint(P + at, make_float4(f2_lo(w[e].x), f2_lo(w[e].y), f2_hi(w[e].x), f2_hi(w[e].y)), keep);
+            }
+        } else if (LG > 0 && rows_layout) {
+            // the column's pairs staged in row order over the exchange area, then scattered
+            float4* const S = reinterpret_cast<float4*>(smraw);
+            const int sw = spec_swap(m);
+#pragma unroll
+            for (int e = 0; e < E / 2; e++)  // crop to N_u rows
+                S[(t + e * NT) ^ sw] = make_float4(f2_lo(w[e].x), f2_lo(w[e].y), f2_hi(w[e].x), f2_hi(w[e].y));
+            sg_fence_proxy_async();
+            __syncthreads();
+            if (t == 0) {
+                SG_IF_OK(m < half && sg_smem_in(smraw, S, (uint32_t)nu * 16), err, 308)
+                spec_store_column(&mapP, m, nu / 2, S, keep);
+                sg_bulk_commit();
+                sg_bulk_wait_read();
+            }
+        } else if constexpr (LG > 0) {
             // the pair layout: {B, C} of each row in 16 bytes (Br holds the pairs)
             float4* P = reinterpret_cast<float4*>(Br) + (size_t)m * nu;
 #pragma unroll
@@ -996,7 +1064,7 @@ __global__ void __launch_bounds__(256) k_edge_bwd(const typename CX<T>::t* __res
                                                   const typename CX<T>::t* __restrict__ C, typename CX<T>::t* B,
                                                   const T* __restrict__ gr, const T* __restrict__ gp,
                                                   const T* __restrict__ wpre, EdgeCoef<T> coef, int nu, int nphi,
-                                                  int ps)
+                                                  int ps, int rows_layout)
 {
     typedef typename CX<T>::t V;
     __shared__ T red[8][8];
@@ -1008,7 +1076,8 @@ __global__ void __launch_bounds__(256) k_edge_bwd(const typename CX<T>::t* __res
     for (int i = threadIdx.x; i < nu; i += blockDim.x) {
         const int idx[4] = {i + 1 + nu, i + nu, i + 1, i};
         const T w = wpre[i];
-        const V a = A[((size_t)m * nu + i) * ps];
+        const size_t at = rows_layout ? spec_at(m, i, half, 1) : (size_t)m * nu + i;
+        const V a = A[at * ps];
         if (m == 0) {
 #pragma unroll
             for (int q = 0; q < 4; q++) {
@@ -1016,7 +1085,7 @@ __global__ void __launch_bounds__(256) k_edge_bwd(const typename CX<T>::t* __res
                 acc[2 * q + 1] += w * gN[idx[q]] * a.y;
             }
         } else {
-            const V c = C[((size_t)m * nu + i) * ps];
+            const V c = C[at * ps];
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const T r = w * g0[idx[q]], p = w * p0[idx[q]];
@@ -1051,8 +1120,9 @@ __global__ void __launch_bounds__(256) k_edge_bwd(const typename CX<T>::t* __res
             dy += coef.c[4 * q + b] * ty[q];
         }
         // the rows b are distinct (N_u >= 4): one thread each
-        V o = B[(size_t)m * nu + brow[b]];
-        B[(size_t)m * nu + brow[b]] = V{o.x + dx, o.y + dy};
+        const size_t at = rows_layout ? spec_at(m, brow[b] ^ (2 * spec_swap(m)), half, 2) : (size_t)m * nu + brow[b];
+        const V o = B[at];
+        B[at] = V{o.x + dx, o.y + dy};
     }
 }
 
@@ -1183,6 +1253,40 @@ __host__ __device__ __forceinline__ size_t bcols_smem_bytes(int nu)
     return sg_align16(sg_padded(L) * sizeof(V)) + (size_t)nu * sizeof(V) + 2 * (size_t)KS * sizeof(V);
 }
 
+// Y = X_a conj(Khat_r) + X_c conj(Khat_phi) at a thread's frequencies (X_a, X_c
+// paired in w); sm: a free exchange area.  Every thread of the block calls.
+template <int E>
+__device__ __forceinline__ void bwd_cols_products(const C2 (&w)[E], float2* sm, const float2* kr_s, const float2* kp_s,
+                                                  int m, int t, int nu, float2 (&y)[E])
+{
+    typedef float2 V;
+    typedef float T;
+    const int L = 2 * nu, NT = L / E;
+    if (m == 0) {
+        // X_a is the FFT of (DC + i Nyquist); the phi kernel vanishes at
+        // modes 0 and N_phi/2, so X_c is not needed
+#pragma unroll
+        for (int e = 0; e < E; e++) sm[sg_pad(t + e * NT)] = c2_lo(w[e]);
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; e++) {
+            const int k = t + e * NT;
+            const V z = c2_lo(w[e]), zc = cconj(sm[sg_pad((L - k) & (L - 1))]);
+            const V a = cscale(cadd(z, zc), (T)0.5);
+            const V d = csub(z, zc);
+            const V b = V{d.y * (T)0.5, -d.x * (T)0.5};
+            y[e] = cadd(cmul(a, cconj(khat_r_s(kr_s, k, L, nu))), cmuli(cmul(b, cconj(khat_r_s(kp_s, k, L, nu)))));
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; e++) {
+            V a, b;
+            khat_at<E>(kr_s, kp_s, t, e, NT, a, b);
+            y[e] = cadd(cmul(c2_lo(w[e]), cconj(a)), cmul(c2_hi(w[e]), cconj(b)));
+        }
+    }
+}
+
 // EDGE (FP32, 16 points per thread, L >= 512): the transposed edge-slope
 // update of k_edge_bwd is applied here: the mode's rows of the edge tables
 // arrive with the spectra (into the exchange area, which is free until the
@@ -1198,7 +1302,9 @@ __global__ void SG_COLS_BOUNDS(T, NTB) k_bwd_cols(const typename CX<T>::t* __res
                                                   typename CX<T>::t* __restrict__ B, int nu, int nphi, int log2L,
                                                   const typename CX<T>::t* __restrict__ tw, int* err,
                                                   const T* __restrict__ egr, const T* __restrict__ egp,
-                                                  const T* __restrict__ wpre, EdgeCoef<T> ecoef)
+                                                  const T* __restrict__ wpre, EdgeCoef<T> ecoef,
+                                                  const __grid_constant__ CUtensorMap mapP,
+                                                  const __grid_constant__ CUtensorMap mapB, int rows_layout)
 {
     const unsigned long long wlim = sg_wait_budget(err);  // read once, early
     if constexpr (LG > 0) {  // the length is a compile-time constant
@@ -1252,8 +1358,12 @@ __global__ void SG_COLS_BOUNDS(T, NTB) k_bwd_cols(const typename CX<T>::t* __res
         if constexpr (pairs) {
             sg_mbar_expect_tx(&bar[0], 2 * ab);
             SG_IF_OK(sg_in((long long)2 * m * nu, 2 * nu, (long long)2 * half * nu) && sg_smem_in(smraw, sm, 2 * ab),
-                     err, 401)
-            sg_bulk_g2s_hint(sm, A + (size_t)2 * m * nu, 2 * ab, &bar[0], drop);
+                     err, 401) {
+                if (rows_layout)
+                    spec_load_column(sm, &mapP, m, nu / 2, &bar[0], drop);
+                else
+                    sg_bulk_g2s_hint(sm, A + (size_t)2 * m * nu, 2 * ab, &bar[0], drop);
+            }
         } else {
             sg_mbar_expect_tx(&bar[0], ab);
             SG_IF_OK(sg_in((long long)m * nu, nu, (long long)half * nu) && sg_smem_in(smraw, sm, ab) &&
@@ -1321,29 +1431,7 @@ __global__ void SG_COLS_BOUNDS(T, NTB) k_bwd_cols(const typename CX<T>::t* __res
         // rows >= N_u are zero; the transform's first exchange waits for the landing reads
         sg_fft_pair<-1, LG, true>(w, reinterpret_cast<C2*>(smraw), L, log2L, t, twd.h);
         V y[E];
-        if (m == 0) {
-            // X_a is the FFT of (DC + i Nyquist); the phi kernel vanishes at
-            // modes 0 and N_phi/2, so X_c is not needed
-#pragma unroll
-            for (int e = 0; e < E; e++) sm[sg_pad(t + e * NT)] = c2_lo(w[e]);
-            __syncthreads();
-#pragma unroll
-            for (int e = 0; e < E; e++) {
-                const int k = t + e * NT;
-                const V z = c2_lo(w[e]), zc = cconj(sm[sg_pad((L - k) & (L - 1))]);
-                const V a = cscale(cadd(z, zc), (T)0.5);
-                const V d = csub(z, zc);
-                const V b = V{d.y * (T)0.5, -d.x * (T)0.5};
-                y[e] = cadd(cmul(a, cconj(khat_r_s(kr_s, k, L, nu))), cmuli(cmul(b, cconj(khat_r_s(kp_s, k, L, nu)))));
-            }
-        } else {
-#pragma unroll
-            for (int e = 0; e < E; e++) {
-                V a, b;
-                khat_at<E>(kr_s, kp_s, t, e, NT, a, b);
-                y[e] = cadd(cmul(c2_lo(w[e]), cconj(a)), cmul(c2_hi(w[e]), cconj(b)));
-            }
-        }
+        bwd_cols_products<E>(w, sm, kr_s, kp_s, m, t, nu, y);
         fft<E, +1, LG>(y, sm, L, log2L, t, twd);  // waits for the mirror reads
         if constexpr (EDGE) {
             // rows 0, 1 are element 0 of threads 0, 1; rows N_u-2, N_u-1 element
@@ -1363,6 +1451,31 @@ __global__ void SG_COLS_BOUNDS(T, NTB) k_bwd_cols(const typename CX<T>::t* __res
             };
             if (t < 2) y[0] = cadd(y[0], update(t));
             if (t >= NT - 2) y[E / 2 - 1] = cadd(y[E / 2 - 1], update(t - NT + 4));
+        }
+        if (LG > 12 && rows_layout) {  // as the forward pass
+            const int sw = 2 * spec_swap(m);
+#pragma unroll
+            for (int e = 0; e < E / 2; e++) {
+                const size_t at = spec_at(m, (t + e * NT) ^ sw, half, 2);
+                SG_IF_OK(sg_in((long long)at, 1, (long long)half * nu), err, 408)
+                sg_st_hint(B + at, y[e], keep);
+            }
+            return;
+        }
+        if (LG > 0 && rows_layout) {
+            // staged in row order (the transform's last exchange is read), then scattered
+            const int sw = 2 * spec_swap(m);
+#pragma unroll
+            for (int e = 0; e < E / 2; e++) sm[(t + e * NT) ^ sw] = y[e];
+            sg_fence_proxy_async();
+            __syncthreads();
+            if (t == 0) {
+                SG_IF_OK(m < half && sg_smem_in(smraw, sm, ab), err, 407)
+                spec_store_column(&mapB, m, nu / 4, sm, keep);
+                sg_bulk_commit();
+                sg_bulk_wait_read();
+            }
+            return;
         }
 #pragma unroll
         for (int e = 0; e < E / 2; e++)
@@ -1620,10 +1733,7 @@ __global__ void __launch_bounds__(512) k_spec_cols(const double2* __restrict__ W
 
 // ===========================================================================
 // FP32 row passes with the transform length N = 2^LG fixed at compile time,
-// moving the mode-major spectra in whole 32-byte L2 sectors.  A copy of
-// 16-byte pieces (one mode of two FP32 complex rows) runs at half the rate
-// of 32-byte ones, on the TMA unit and the load-store path alike, so every
-// thread or stage row here carries four complex values of one mode.
+// on the row layout: a unit of rows is one contiguous piece of its spectra.
 //
 // One block per unit of rows: TPG = GT / (N/16) paired transforms
 // (sg_fft_pair: two complex FFTs in lockstep on the f32x2 instructions) of
@@ -1639,18 +1749,15 @@ __global__ void __launch_bounds__(512) k_spec_cols(const double2* __restrict__ W
 //    A[m][i0..i0+3] (8 bytes each) leave in one 256-bit store.  Adjoint
 //    (P1b): z1 = wpost_i0 (gF_r + i gF_phi)_i0, z2 for i0+1; the (A, C)
 //    pairs of both rows leave in one 256-bit store.
-//  k_rows_c2r<LG, BWD>: per transform one paired inverse FFT, staged by
-//    tensor copies whose box rows are 32 bytes (one mode of the transform's
-//    rows), stored with the 32-byte swizzle so that the stage reads are free
-//    of bank conflicts.  Forward (P3): rows (i0, i0+1) of the (B, C) pairs,
-//    Z = B + i C each; F_r, F_phi = Re, Im Z times wpost.  Adjoint (P3b):
-//    rows i0..i0+3 of B, Z = S_i0 + i S_i0+1 and S_i0+2 + i S_i0+3; gsigma
-//    = Re, Im times wpre.
+//  k_rows_c2r<LG, BWD>: per transform one paired inverse FFT of the unit's
+//    spectra, one bulk copy.  Forward (P3): rows (i0, i0+1) of the (B, C)
+//    pairs, Z = B + i C each; F_r, F_phi = Re, Im Z times wpost.  Adjoint
+//    (P3b): rows i0..i0+3 of B, Z = S_i0 + i S_i0+1 and S_i0+2 + i S_i0+3;
+//    gsigma = Re, Im times wpre.
 //
-// The pair layout P keeps two complex values per (mode, row) in 16 bytes:
-// P[m nu + i] = {X_i, Y_i}, m < N_phi/2 (forward X = B, Y = C; adjoint
-// X = A, Y = C); the single layout S[m nu + i] keeps one (forward A,
-// adjoint B).  Mode 0 packs (DC, Nyquist) in both.
+// Pairs keep two complex values per (mode, row) in 16 bytes, {X_i, Y_i}
+// (forward X = B, Y = C; adjoint X = A, Y = C); single values are the
+// forward's A and the adjoint's B.  Mode 0 packs (DC, Nyquist) in both.
 // ===========================================================================
 // blocks per SM the fixed-length row passes' registers are bounded for
 // (3: 80 registers, the shared memory of three 70 KB areas)
@@ -1805,13 +1912,13 @@ __device__ __forceinline__ bool rows_r2c_unit(const float* __restrict__ x0, cons
     sg_fft_pair<-1, LG>(w, sm, N, LG, t, twd.h, bsync);
     C2 xa[8], xb[8];
     split_real_pair2(w, sm, N, t, xa, xb, bsync);
-    // forward: A[m][i0..i0+3]; adjoint: {A, C} of rows i0, i0+1 (32 bytes, aligned)
+    // forward: A of rows i0..i0+3; adjoint: {A, C} of rows i0, i0+1: one unit a mode
     const uint64_t keep = sg_policy_evict_last();  // the column pass reads the spectra from L2
 #pragma unroll
     for (int e = 0; e < 8; e++) {
-        const size_t mi = (size_t)(t + e * NT) * nu + i0;
-        float* q = reinterpret_cast<float*>(out) + (BWD ? 4 : 2) * mi;
-        SG_IF_OK(sg_in((long long)mi, BWD ? 2 : 4, (long long)(N / 2) * nu), err, 103)
+        const size_t unit = (size_t)(i0 / RPT) * (N / 2) + t + e * NT;
+        float* q = reinterpret_cast<float*>(out) + 8 * unit;
+        SG_IF_OK(sg_in((long long)unit, 1, (long long)(N / 2) * (nu / RPT)), err, 103)
         sg_st256_hint(q, make_float4(f2_lo(xa[e].x), f2_lo(xa[e].y), f2_lo(xb[e].x), f2_lo(xb[e].y)),
                       make_float4(f2_hi(xa[e].x), f2_hi(xa[e].y), f2_hi(xb[e].x), f2_hi(xb[e].y)), keep);
     }
@@ -1835,7 +1942,7 @@ __global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MI
 // One unit of the row C2R pass (rows u R .. u R + R - 1), shared like
 // rows_r2c_unit; map: the tensor map in kernel-parameter or global memory.
 template <int LG, bool BWD, bool PDL, bool SMALL = false>
-__device__ __forceinline__ bool rows_c2r_unit(const CUtensorMap* map, const float* __restrict__ wrow,
+__device__ __forceinline__ bool rows_c2r_unit(const float4* in, const float* __restrict__ wrow,
                                               float* __restrict__ y0, float* __restrict__ y1, int nu,
                                               const float2* __restrict__ tw, int* err, int u, unsigned char* smraw,
                                               uint64_t& bar, uint32_t phase, unsigned long long wlim,
@@ -1845,8 +1952,7 @@ __device__ __forceinline__ bool rows_c2r_unit(const CUtensorMap* map, const floa
     constexpr int N = RU::N, NT = RU::NT, TPG = RU::TPG, half = N / 2;
     constexpr int RPT = BWD ? 4 : 2;  // rows per transform
     constexpr int R = RPT * TPG;      // rows per block
-    constexpr int MB = half < 256 ? half : 256, NBOX = half / MB;
-    unsigned char* const area = align_smem<1024>(smraw);  // the swizzle repeats every 256 bytes
+    unsigned char* const area = align128(smraw);
     const int tr = threadIdx.x / NT, t = threadIdx.x % NT;
     const int i0 = u * R + tr * RPT;
     const Twd<16, float2> twd = make_twd<16>(LG, t, tw);
@@ -1862,26 +1968,19 @@ __device__ __forceinline__ bool rows_c2r_unit(const CUtensorMap* map, const floa
         sg_grid_dep_launch();
         sg_grid_dep_wait();  // the spectra are the previous pass's results
     }
-    if (threadIdx.x < 32) {
+    if (threadIdx.x == 0) {
         // transform j's rows land at j N x 16 bytes, mode n of them at 32 n
-        const int lane = threadIdx.x;
-        if (lane == 0) sg_mbar_expect_tx(&bar, (uint32_t)(TPG * half * 32));
-        __syncwarp();
-        const uint64_t drop = sg_policy_evict_first();  // the spectra are consumed here
-        for (int j = lane; j < TPG * NBOX; j += 32) {
-            const int s = j / NBOX, b = j % NBOX;
-            const int x = (BWD ? 1 : 2) * (u * R + s * RPT);  // 8-byte units: x even keeps the 16-byte rule
-            SG_IF_OK((x & 1) == 0 && sg_in(x, 4, (BWD ? 1 : 2) * (long long)nu) && sg_in(b * MB, MB, half) &&
-                         sg_smem_in(smraw, area + (size_t)s * N * 16 + (size_t)b * MB * 32, MB * 32),
-                     err, 202)
-            sg_tma_load_2d(area + (size_t)s * N * 16 + (size_t)b * MB * 32, map, x, b * MB, &bar, drop);
-        }
+        constexpr uint32_t bytes = (uint32_t)(TPG * half * 32);
+        sg_mbar_expect_tx(&bar, bytes);
+        const long long unit = (long long)u * TPG * half;
+        SG_IF_OK(sg_in(unit, TPG * half, (long long)half * (nu / RPT)) && sg_smem_in(smraw, area, bytes), err, 202)
+        sg_bulk_g2s_hint(area, in + 2 * unit, bytes, &bar, sg_policy_evict_first());  // consumed here
     }
     if (__syncthreads_or(!sg_mbar_wait_bounded(&bar, phase, err, 1, wlim, landed))) return false;  // inputs never arrived
     const float4* const S4 = reinterpret_cast<const float4*>(area) + (size_t)tr * N;  // this transform's modes
-    // Z of both lanes at frequency n.  Each mode holds two 16-byte units u0,
+    // Z of both lanes at frequency n.  Each mode holds two 16-byte halves u0,
     // u1 (forward: {B, C} of rows i0, i0+1; adjoint: {S_i0, S_i0+1}, {S_i0+2,
-    // S_i0+3}), the halves of modes with bit 2 set swapped by the swizzle.
+    // S_i0+3}), swapped for modes with bit 2 set.
     // With u = (p.x, p.y, q.x, q.y): Z = p + i q below N/2 and conj p + i
     // conj q above (q of mode 0 vanishes in the forward direction: the
     // azimuthal kernel is odd)
@@ -1890,7 +1989,7 @@ __device__ __forceinline__ bool rows_c2r_unit(const CUtensorMap* map, const floa
     for (int e = 0; e < 16; e++) {
         const int n = t + e * NT;
         const int mo = e < 8 ? n : (n == half ? 0 : N - n);  // n = N/2 reads mode 0 (Nyquist)
-        const int sw = (mo >> 2) & 1;
+        const int sw = spec_swap(mo);
         const float4 u0 = S4[2 * mo + sw], u1 = S4[2 * mo + (sw ^ 1)];
         if (n == 0)
             w[e] = C2{f2(u0.x, u1.x), f2(u0.z, u1.z)};
@@ -1928,12 +2027,10 @@ __device__ __forceinline__ bool rows_c2r_unit(const CUtensorMap* map, const floa
     return true;
 }
 
-// map: 2-D tensor map over the input (forward: the pair layout, two 8-byte
-// units per row; adjoint: the single layout, one unit per row) with boxes
-// of 4 units x min(N/2, 256) modes and the 32-byte swizzle
+// in: the input spectra (forward: the pairs; adjoint: the single values)
 template <int LG, bool BWD, bool SMALL = false>
 __global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MINB)
-    k_rows_c2r(const __grid_constant__ CUtensorMap map, const float* __restrict__ wrow, float* __restrict__ y0,
+    k_rows_c2r(const float4* in, const float* __restrict__ wrow, float* __restrict__ y0,
                float* __restrict__ y1, int nu, const float2* __restrict__ tw, int* err)
 {
     const unsigned long long wlim = sg_wait_budget(err);  // read once, early
@@ -1941,7 +2038,138 @@ __global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MI
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) sg_mbar_init(&bar, 1);
     __syncthreads();
-    rows_c2r_unit<LG, BWD, true, SMALL>(&map, wrow, y0, y1, nu, tw, err, blockIdx.x, smraw, bar, 0, wlim);
+    rows_c2r_unit<LG, BWD, true, SMALL>(in, wrow, y0, y1, nu, tw, err, blockIdx.x, smraw, bar, 0, wlim);
+}
+
+// ===========================================================================
+// The column passes for 8192 points (N_u = 4096), whose exchange area leaves
+// room for one block per SM: nothing else hides a block's copies there, so the
+// blocks are persistent and one 64 KB buffer beside the exchange area takes,
+// in turn, a mode's column (while the previous mode's inverse transform runs)
+// and its two spectrum rows (while its forward transform runs).  Results leave
+// by each thread's own stores.  N_u x N_phi = 4096 x 8192, one block per mode ->
+// persistent, us: forward 365 -> 302, adjoint 373 -> 292.
+// ===========================================================================
+// the buffer's place: after the exchange area, 128-byte aligned for tensor copies
+__host__ __device__ __forceinline__ size_t ring_cols_buffer(int nu) { return (sg_padded(2 * nu) * sizeof(C2) + 127) & ~(size_t)127; }
+__host__ __device__ __forceinline__ size_t ring_cols_smem_bytes(int nu)
+{
+    return ring_cols_buffer(nu) + 2 * (size_t)(nu + 2) * sizeof(float2);
+}
+// a block barrier whose first call also runs fn on thread 0, once every
+// thread has arrived
+template <typename F>
+struct SgSyncThen {
+    F fn;
+    mutable bool done = false;
+    __device__ __forceinline__ explicit SgSyncThen(F f) : fn(f) {}
+    __device__ __forceinline__ void operator()() const
+    {
+        __syncthreads();
+        if (!done && threadIdx.x == 0) fn();
+        done = true;
+    }
+};
+
+template <int LG, bool BWD>
+__global__ void __launch_bounds__((1 << LG) / 16, 1)
+    k_ring_cols(const float2* __restrict__ Kr, const float2* __restrict__ Kp, float2* __restrict__ out, int half,
+                const float2* __restrict__ tw, int* err, const __grid_constant__ CUtensorMap map, const float2* in,
+                int rows_layout)
+{
+    constexpr int L = 1 << LG, nu = L / 2, NT = L / 16, KS = nu + 2;
+    constexpr uint32_t ab = nu * (BWD ? 16 : 8), kb = KS * 8;
+    const unsigned long long wlim = sg_wait_budget(err);  // read once, early
+    extern __shared__ __align__(128) unsigned char smraw[];
+    __shared__ __align__(8) uint64_t bar[2];  // [0]: columns, [1]: spectra
+    const int t = threadIdx.x;
+    float2* const sm = reinterpret_cast<float2*>(smraw);
+    unsigned char* const buf = smraw + ring_cols_buffer(nu);
+    if (t == 0) {
+        sg_mbar_init(&bar[0], 1);
+        sg_mbar_init(&bar[1], 1);
+    }
+    __syncthreads();
+    const Twd<16, float2> twd = make_twd<16>(LG, t, tw);
+    const uint64_t drop = sg_policy_evict_first(), keep = sg_policy_evict_last();
+    // thread 0, with the buffer free
+    const auto issue_column = [&](int m) {
+        sg_fence_proxy_async();
+        sg_mbar_expect_tx(&bar[0], ab);
+        SG_IF_OK(m < half && sg_smem_in(smraw, buf, ab), err, 321) {
+            if (rows_layout)
+                spec_load_column(buf, &map, m, nu / (BWD ? 2 : 4), &bar[0], drop);
+            else
+                sg_bulk_g2s_hint(buf, reinterpret_cast<const unsigned char*>(in) + (size_t)m * ab, ab, &bar[0], drop);
+        }
+    };
+    const auto issue_spectra = [&](int m) {
+        sg_fence_proxy_async();
+        sg_mbar_expect_tx(&bar[1], 2 * kb);
+        SG_IF_OK(m < half && sg_smem_in(smraw, buf, 2 * kb), err, 322) {
+            sg_bulk_g2s_hint(buf, Kr + (size_t)m * KS, kb, &bar[1], drop);
+            // mode 0 holds (DC, Nyquist): the Nyquist mode's Khat_r instead of Khat_phi
+            sg_bulk_g2s_hint(buf + kb, (m == 0 ? Kr + (size_t)half * KS : Kp + (size_t)m * KS), kb, &bar[1], drop);
+        }
+    };
+    sg_grid_dep_launch();
+    sg_grid_dep_wait();  // the columns are the previous pass's results
+    if (t == 0) issue_column(blockIdx.x);
+    uint32_t ph = 0;
+    for (int m = blockIdx.x; m < half; m += gridDim.x, ph ^= 1) {
+        const int next = m + gridDim.x;
+        if (__syncthreads_or(!sg_mbar_wait_bounded(&bar[0], ph, err, 1, wlim))) return;  // the column never arrived
+        const float2* const kr_s = reinterpret_cast<const float2*>(buf);
+        const float2* const kp_s = kr_s + KS;
+        const auto wait_spectra = [&] { return !__syncthreads_or(!sg_mbar_wait_bounded(&bar[1], ph, err, 1, wlim)); };
+        // once the spectra are read (the inverse transforms' first barrier) the buffer takes the next column
+        const auto then_next = [&] {
+            if (next < half) issue_column(next);
+        };
+        const SgSyncThen<decltype(then_next)> isync(then_next);
+        const int sw = spec_swap(m);
+        if constexpr (!BWD) {
+            float2 v[16];
+#pragma unroll
+            for (int e = 0; e < 16; e++)
+                v[e] = e < 8 ? reinterpret_cast<const float2*>(buf)[t + e * NT] : float2{0.f, 0.f};  // zero pad
+            __syncthreads();  // the column is read
+            if (t == 0) issue_spectra(m);
+            C2 w[16];
+            if (!fwd_cols_math<LG, false>(v, sm, kr_s, kp_s, reinterpret_cast<C2*>(smraw), m, t, nu, LG, twd,
+                                          wait_spectra, w, isync))
+                return;
+            float4* const P = reinterpret_cast<float4*>(out);
+#pragma unroll
+            for (int e = 0; e < 8; e++) {  // crop to N_u rows
+                const int i = t + e * NT;
+                const size_t at = rows_layout ? spec_at(m, i ^ sw, half, 1) : (size_t)m * nu + i;
+                SG_IF_OK(sg_in((long long)at, 1, (long long)half * nu), err, 323)
+                sg_st_hint(P + at, make_float4(f2_lo(w[e].x), f2_lo(w[e].y), f2_hi(w[e].x), f2_hi(w[e].y)), keep);
+            }
+        } else {
+            C2 w[16];
+#pragma unroll
+            for (int e = 0; e < 16; e++) {
+                const float4 u = e < 8 ? reinterpret_cast<const float4*>(buf)[t + e * NT] : make_float4(0.f, 0.f, 0.f, 0.f);
+                w[e] = C2{f2(u.x, u.z), f2(u.y, u.w)};
+            }
+            __syncthreads();
+            if (t == 0) issue_spectra(m);
+            sg_fft_pair<-1, LG, true>(w, reinterpret_cast<C2*>(smraw), L, LG, t, twd.h);
+            if (!wait_spectra()) return;
+            float2 y[16];
+            bwd_cols_products<16>(w, sm, kr_s, kp_s, m, t, nu, y);
+            fft<16, +1, LG>(y, sm, L, LG, t, twd, isync);
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const int i = t + e * NT;
+                const size_t at = rows_layout ? spec_at(m, i ^ (2 * sw), half, 2) : (size_t)m * nu + i;
+                SG_IF_OK(sg_in((long long)at, 1, (long long)half * nu), err, 324)
+                sg_st_hint(out + at, y[e], keep);
+            }
+        }
+    }
 }
 
 // ===========================================================================
@@ -1958,12 +2186,16 @@ __global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MI
 // the pass kernels' signatures (spelled out: naming an instance here would
 // refer to kernels that each translation unit does not define)
 typedef void (*RowsR2CFn)(const float*, const float*, const float*, float2*, int, const float2*, int*, int);
-typedef void (*RowsC2RFn)(CUtensorMap, const float*, float*, float*, int, const float2*, int*);
+typedef void (*RowsC2RFn)(const float4*, const float*, float*, float*, int, const float2*, int*);
 typedef void (*FwdColsFn)(const float2*, const float2*, const float2*, float2*, float2*, int, int, int,
                           const float2*, int*, const float*, const float*, const float*, EdgeCoef<float>,
-                          WedgeArgs<float>);
+                          WedgeArgs<float>, CUtensorMap, CUtensorMap, int);
 typedef void (*BwdColsFn)(const float2*, const float2*, const float2*, const float2*, float2*, int, int, int,
-                          const float2*, int*, const float*, const float*, const float*, EdgeCoef<float>);
+                          const float2*, int*, const float*, const float*, const float*, EdgeCoef<float>,
+                          CUtensorMap, CUtensorMap, int);
+
+typedef void (*RingColsFn)(const float2*, const float2*, float2*, int, const float2*, int*, CUtensorMap, const float2*,
+                           int);
 
 struct FixedRowKernels {
     RowsR2CFn fwd_rows;         // k_rows_r2c, forward
@@ -1982,6 +2214,7 @@ struct FixedPassKernels {
     FwdColsFn fwd_cols_edge_wedge;  // with the edge-slope and origin-wedge updates
     BwdColsFn bwd_cols;
     BwdColsFn bwd_cols_edge;  // with the transposed edge-slope update
+    RingColsFn ring_cols[2];  // k_ring_cols, forward and adjoint, or null (lengths below 8192)
     // the row instances for passes of `rows_per_transform` rows each: the small
     // blocks while the others are fewer than the SMs
     const FixedRowKernels& pick(int nu, int rows_per_transform, int sms) const
@@ -1999,6 +2232,14 @@ FixedRowKernels make_fixed_row_kernels()
                            k_rows_c2r<LG, true, SMALL>,        RU::SMEM,
                            RU::GT,                             RU::TPG};
 }
+template <int LG, bool BWD>
+RingColsFn ring_cols_kernel()
+{
+    if constexpr (LG > 12)
+        return k_ring_cols<LG, BWD>;
+    else
+        return nullptr;
+}
 template <int LG>
 FixedPassKernels make_fixed_pass_kernels()
 {
@@ -2009,7 +2250,8 @@ FixedPassKernels make_fixed_pass_kernels()
                             k_fwd_cols<float, 16, NB, LG, true>,
                             k_fwd_cols<float, 16, NB, LG, true, true>,
                             k_bwd_cols<float, 16, NB, LG>,
-                            k_bwd_cols<float, 16, NB, LG, true>};
+                            k_bwd_cols<float, 16, NB, LG, true>,
+                            {ring_cols_kernel<LG, false>(), ring_cols_kernel<LG, true>()}};
 }
 
 // defined in fftconv_lg<LG>.cu
@@ -2143,16 +2385,16 @@ void make_row_maps(int nu, int nphi, size_t elem, void* const bufs[3], SgRowMaps
 bool make_pair_maps(int nu, int nphi, void* wa, void* wb, CUtensorMap out[2])
 {
     EncodeTiledFn enc = tensor_map_encoder();
-    if (!enc || nphi < 32) return false;
-    const int half = nphi / 2, MB = row_box_modes(half);
+    if (!enc || nphi < 32 || nu < 4) return false;
+    const int half = nphi / 2;
     for (int k = 0; k < 2; k++) {
-        const int c = k == 0 ? 2 : 1;  // 8-byte units per row: (X, Y) pairs, single values
-        const cuuint64_t dims[2] = {(cuuint64_t)c * nu, (cuuint64_t)half};
-        const cuuint64_t strides[1] = {(cuuint64_t)c * nu * 8};
-        const cuuint32_t box[2] = {4, (cuuint32_t)MB};
-        const cuuint32_t estr[2] = {1, 1};
-        if (enc(&out[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, k == 0 ? wb : wa, dims, strides, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+        const int groups = nu / (k == 0 ? 2 : 4);  // rows per 32-byte unit: two pairs, four single values
+        const cuuint64_t dims[3] = {4, (cuuint64_t)half, (cuuint64_t)groups};
+        const cuuint64_t strides[2] = {32, (cuuint64_t)half * 32};
+        const cuuint32_t box[3] = {4, 1, (cuuint32_t)spec_box_rows(groups)};
+        const cuuint32_t estr[3] = {1, 1, 1};
+        if (enc(&out[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, k == 0 ? wb : wa, dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return false;
     }
@@ -2197,7 +2439,7 @@ static cudaError_t launch_edges(const PlanView& p, bool adjoint, cudaStream_t st
     if (adjoint)
         k_edge_bwd<T><<<p.nphi / 2, 256, 0, st>>>(p.pairs ? X : (const V*)p.wa, Y, p.pairs ? (V*)p.wa : X,
                                                   (const T*)p.egr, (const T*)p.egp, (const T*)p.wpre, coef, p.nu,
-                                                  p.nphi, ps);
+                                                  p.nphi, ps, p.pairs == 2);
     else
         k_edge_fwd<T><<<p.nphi / 2, 256, 0, st>>>((const V*)p.wa, X, Y, (const T*)p.egr, (const T*)p.egp,
                                                   (const T*)p.wpre, coef, p.nu, p.nphi, ps);
@@ -2225,6 +2467,29 @@ static bool fixed_path(const PlanView& p, const FixedPassKernels*& fr, const Fix
     return true;
 }
 
+// The persistent column passes: one block per SM, each taking every grid-th
+// mode.  Not for at most one mode per SM, where k_fwd_cols copies the spectra
+// before the row pass ends (4096 x 32 forward: 21.0 against 22.6 us), and not
+// with edge tables, for which the buffer leaves no room.
+static bool ring_cols_fit(const PlanView& p, const FixedPassKernels* fc)
+{
+    return p.pairs && !p.edges && fc->ring_cols[0] && p.nphi / 2 > p.sms;
+}
+static cudaError_t launch_ring_cols(const PlanView& p, RingColsFn k, bool adjoint, cudaStream_t st)
+{
+    const size_t smem = ring_cols_smem_bytes(p.nu);
+    cudaError_t err = set_smem(k, smem, true);
+    if (err != cudaSuccess) return err;
+    const int half = p.nphi / 2;
+    float2* const single = (float2*)p.wa;
+    float2* const pairs = (float2*)p.wb;
+    const CUtensorMap none{};
+    return launch_pdl(k, half < p.sms ? half : p.sms, 2 * p.nu / 16, smem, st, (const float2*)p.kr,
+                      (const float2*)p.kp, adjoint ? single : pairs, half, (const float2*)p.tw, p.err,
+                      p.pairs == 2 ? p.imaps[adjoint ? 0 : 1] : none, (const float2*)(adjoint ? pairs : single),
+                      p.pairs == 2);
+}
+
 template <typename T>
 cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cudaStream_t st, cudaEvent_t* ev,
                            bool sigma_direct)
@@ -2232,7 +2497,7 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
     typedef typename CX<T>::t V;
     const FixedPassKernels *fr, *fc;
     PlanView p = p0;
-    p.pairs = fixed_path<T>(p0, fr, fc) ? 1 : 0;
+    p.pairs = !fixed_path<T>(p0, fr, fc) ? 0 : p.tcm ? 1 : 2;
     const V* tw = (const V*)p.tw;
     V* A = (V*)p.wa;
     V* B = (V*)p.wb;
@@ -2283,6 +2548,9 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
     if (std::is_same<T, double>::value && fx_cols_ok(p)) {
         PassRange range_("sg forward columns");
         if ((err = launch_fx_cols(p, false, st)) != cudaSuccess) return err;
+    } else if (ring_cols_fit(p, fc)) {
+        PassRange range_("sg forward columns");
+        if ((err = launch_ring_cols(p, fc->ring_cols[0], false, st)) != cudaSuccess) return err;
     } else {
         PassRange range_("sg forward columns");
         const int L = 2 * p.nu, E = L >= 16 ? 16 : L;
@@ -2307,7 +2575,8 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
             if ((err = set_smem(k, smem, true)) != cudaSuccess) return err;
             if ((err = launch_pdl(k, p.nphi / 2, L / EE, smem, st, A, (const V*)p.kr, (const V*)p.kp, B, C, p.nu,
                                   p.nphi, lL, tw, p.err, (const T*)p.egr, (const T*)p.egp, (const T*)p.wpre,
-                                  coef, wdg)) != cudaSuccess)
+                                  coef, wdg, p.pairs == 2 ? p.imaps[1] : CUtensorMap{},
+                                  p.pairs == 2 ? p.imaps[0] : CUtensorMap{}, p.pairs == 2)) != cudaSuccess)
                 return err;
             edges_done = fuse;
         });
@@ -2324,7 +2593,7 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
             const int nblk = p.nu / (2 * rk.slots);
             auto k = rk.fwd_rows_inv;
             if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
-            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, p.imaps[0], (const float*)p.wpost, (float*)Fr, (float*)Fp, p.nu,
+            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, (const float4*)p.wb, (const float*)p.wpost, (float*)Fr, (float*)Fp, p.nu,
                                   (const float2*)p.tw, p.err)) != cudaSuccess)
                 return err;
         } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
@@ -2358,7 +2627,7 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
     typedef typename CX<T>::t V;
     const FixedPassKernels *fr, *fc;
     PlanView p = p0;
-    p.pairs = fixed_path<T>(p0, fr, fc) ? 1 : 0;
+    p.pairs = !fixed_path<T>(p0, fr, fc) ? 0 : p.tcm ? 1 : 2;
     const V* tw = (const V*)p.tw;
     V* A = (V*)p.wa;
     V* B = (V*)p.wb;
@@ -2404,6 +2673,9 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
     if (std::is_same<T, double>::value && fx_cols_ok(p)) {
         PassRange range_("sg adjoint columns");
         if ((err = launch_fx_cols(p, true, st)) != cudaSuccess) return err;
+    } else if (ring_cols_fit(p, fc)) {
+        PassRange range_("sg adjoint columns");
+        if ((err = launch_ring_cols(p, fc->ring_cols[1], true, st)) != cudaSuccess) return err;
     } else {
         PassRange range_("sg adjoint columns");
         const int L = 2 * p.nu, E = L >= 16 ? 16 : L;
@@ -2424,7 +2696,9 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
             // the pair layout: the (A, C) pairs in wb, B into wa
             if ((err = launch_pdl(k, p.nphi / 2, L / EE, smem, st, p.pairs ? B : A, C, (const V*)p.kr,
                                   (const V*)p.kp, p.pairs ? A : B, p.nu, p.nphi, lL, tw, p.err, (const T*)p.egr,
-                                  (const T*)p.egp, (const T*)p.wpre, coef)) != cudaSuccess)
+                                  (const T*)p.egp, (const T*)p.wpre, coef,
+                                  p.pairs == 2 ? p.imaps[0] : CUtensorMap{},
+                                  p.pairs == 2 ? p.imaps[1] : CUtensorMap{}, p.pairs == 2)) != cudaSuccess)
                 return err;
             edges_done = fuse;
         });
@@ -2441,7 +2715,7 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
             const int nblk = p.nu / (4 * rk.slots);
             auto k = rk.bwd_rows_inv;
             if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
-            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, p.imaps[1], (const float*)p.wpre, (float*)gs, (float*)nullptr,
+            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, (const float4*)p.wa, (const float*)p.wpre, (float*)gs, (float*)nullptr,
                                   p.nu, (const float2*)p.tw, p.err)) != cudaSuccess)
                 return err;
         } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {

@@ -525,6 +525,24 @@ __device__ __forceinline__ void sg_tma_store_2d(const CUtensorMap* map, int x, i
                  "r"(x), "r"(y), "r"(sg_smem_u32(src)), "l"(policy)
                  : "memory");
 }
+__device__ __forceinline__ void sg_tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar,
+                                               uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(sg_smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(sg_smem_u32(bar)), "l"(policy)
+        : "memory");
+}
+__device__ __forceinline__ void sg_tma_store_3d(const CUtensorMap* map, int x, int y, int z, const void* src,
+                                                uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group.L2::cache_hint [%0, {%1, %2, %3}], [%4], %5;" ::"l"(
+            reinterpret_cast<uint64_t>(map)),
+        "r"(x), "r"(y), "r"(z), "r"(sg_smem_u32(src)), "l"(policy)
+        : "memory");
+}
 __device__ __forceinline__ void sg_bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // wait until the bulk stores issued by this thread have read their shared memory
 __device__ __forceinline__ void sg_bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
@@ -1137,6 +1155,15 @@ __device__ __forceinline__ void sg_fft_pair(C2 (&v)[16], C2* sm, int N_, int log
 #pragma unroll 1
         for (int p = 0; p < n16; p++) pass(p);
     }
+}
+
+// The row layout of half spectra (fftconv.cu): the place of element (m, i),
+// pairs (lgr = 1: two rows a unit) or single values (lgr = 2: four), and
+// whether mode m's units keep their halves swapped
+__device__ __forceinline__ int spec_swap(int m) { return (m >> 2) & 1; }
+__device__ __forceinline__ size_t spec_at(int m, int i, int half, int lgr)
+{
+    return (((size_t)(i >> lgr) * half + m) << lgr) + (i & ((1 << lgr) - 1));
 }
 
 // launch-shape helpers shared by the host code

@@ -58,8 +58,8 @@ struct sg_plan {
     SgRowMaps maps[2];     // for R = slots and 2 slots rows per row block
     SgRowMaps na_maps[2];  // the same over the allocation-free scratch
     int have_na_maps;
-    // tensor maps of the fixed-length FP32 inverse row passes (make_pair_maps):
-    // [0] over wb in the pair layout, [1] over wa; have_imaps = 0 if none
+    // tensor maps of the fixed-length FP32 column passes (make_pair_maps): [0]
+    // over wb as pairs, [1] over wa; have_imaps = 0 if none
     CUtensorMap imaps[2];
     int have_imaps;
     CUtensorMap na_imaps[2];  // the same over the allocation-free scratch
@@ -105,8 +105,9 @@ struct PlanView {
     int* err;
     const SgRowMaps* maps;  // [2] over wa, wb, wc, or null
     const CUtensorMap* imaps;  // [2] of make_pair_maps over wb (pairs) and wa, or null
-    int pairs;              // set by the launchers: the column spectra are in the pair layout
-                            // (forward: wb holds (B, C); adjoint: wb holds (A, C), wa holds B)
+    int pairs;              // set by the launchers: the column spectra are pairs (forward: wb holds
+                            // (B, C); adjoint: wb holds (A, C), wa holds B), 1: columns contiguous
+                            // (tensor-core rows), 2: the row layout (fftconv.cu)
     int edges;              // one-sided radial edge slopes: egr, egp, ecoef below
     const void* egr;
     const void* egp;
@@ -176,9 +177,9 @@ cudaError_t launch_wedge_dft(const PlanView& p, cudaStream_t st);
 // Tensor maps of the row passes over the buffers bufs[3] (the layout of wa,
 // wb, wc); out[k].R = 0 where a map cannot be made.
 void make_row_maps(int nu, int nphi, size_t elem, void* const bufs[3], SgRowMaps out[2]);
-// Tensor maps of the fixed-length FP32 inverse row passes: out[0] over wb as
-// the pair layout (two 8-byte units per row), out[1] over wa (one unit per
-// row); boxes of 4 units x min(N_phi/2, 256) modes with the 32-byte swizzle.
+// Tensor maps of the fixed-length FP32 column passes over the row layout
+// (32-byte units [row group][mode]): out[0] over wb as pairs (two rows per
+// unit), out[1] over wa (four rows); boxes of one mode x up to 256 groups.
 // False if they cannot be made (the passes then use the run-time instances).
 bool make_pair_maps(int nu, int nphi, void* wa, void* wb, CUtensorMap out[2]);
 // noalloc.cu: the allocation-free entry point's set-up at plan build and load

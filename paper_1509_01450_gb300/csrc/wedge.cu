@@ -127,7 +127,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_wedge_bwd(const typename CX<T>::t* __restrict__ A,
                                                    const typename CX<T>::t* __restrict__ C, typename CX<T>::t* B,
                                                    const T* __restrict__ tab, const T* __restrict__ wpre,
-                                                   typename CX<T>::t* __restrict__ t_out, int nu, int nphi, int ps)
+                                                   typename CX<T>::t* __restrict__ t_out, int nu, int nphi, int ps,
+                                                   int rows_layout)
 {
     typedef typename CX<T>::t V;
     __shared__ T red[8];
@@ -142,14 +143,15 @@ __global__ void __launch_bounds__(256) k_wedge_bwd(const typename CX<T>::t* __re
     T wx = 0, wy = 0, vx = 0, vy = 0;
     for (int i = threadIdx.x; i < nu; i += blockDim.x) {
         const T w = wpre[i];
-        const V a = A[((size_t)m * nu + i) * ps];
+        const size_t at = (rows_layout ? spec_at(m, i, half, 1) : (size_t)m * nu + i) * ps;
+        const V a = A[at];
         if (m == 0) {
             wx += w * Wr[i] * a.x;
             wy += w * WrN[i] * a.y;
             vx += w * Vr[i] * a.x;
             vy += w * VrN[i] * a.y;
         } else {
-            const V c = C[((size_t)m * nu + i) * ps];
+            const V c = C[at];
             // i p c = p (-c.y + i c.x)
             wx += w * (Wr[i] * a.x - Wp[i] * c.y);
             wy += w * (Wr[i] * a.y + Wp[i] * c.x);
@@ -163,10 +165,11 @@ __global__ void __launch_bounds__(256) k_wedge_bwd(const typename CX<T>::t* __re
     vy = blk_sum(vy, red);
     if (threadIdx.x == 0) {
         const T i0 = (T)1 / wpre[0];
-        V b = B[(size_t)m * nu];
+        const size_t at = rows_layout ? spec_at(m, 2 * spec_swap(m), half, 2) : (size_t)m * nu;  // row 0
+        V b = B[at];
         b.x += vx * i0;
         b.y += vy * i0;
-        B[(size_t)m * nu] = b;
+        B[at] = b;
         t_out[m] = V{wx, wy};
     }
 }
@@ -244,7 +247,8 @@ cudaError_t launch_wedge(const PlanView& p, bool adjoint, cudaStream_t st)
     if (adjoint) {
         if (!p.gsigw) return cudaErrorInvalidValue;
         k_wedge_bwd<T><<<p.nphi / 2, 256, 0, st>>>(p.pairs ? X : (const V*)p.wa, Y, p.pairs ? (V*)p.wa : X,
-                                                   (const T*)p.wtab, (const T*)p.wpre, (V*)p.wtmp, p.nu, p.nphi, ps);
+                                                   (const T*)p.wtab, (const T*)p.wpre, (V*)p.wtmp, p.nu, p.nphi, ps,
+                                                   p.pairs == 2);
         k_wedge_idft<T><<<p.nphi, 256, 0, st>>>((const V*)p.wtmp, (const V*)p.tw, (T*)p.gsigw, p.nphi);
     } else {
         if (!p.sigw) return cudaErrorInvalidValue;
