@@ -1294,7 +1294,10 @@ __device__ __forceinline__ void bwd_cols_products(const C2 (&w)[E], float2* sm, 
 // columns, and the owners of rows 0, 1, N_u-2, N_u-1 add
 // sum_a coef[a][b] t_a before their stores.  egr, egp, wpre and ecoef are
 // unused otherwise.
-template <typename T, int E, int NTB, int LG = 0, bool EDGE = false>
+// WEDGE (with EDGE): the transposed wedge update of k_wedge_bwd likewise, its
+// table rows read straight from global memory: row 0 takes the V part, t_out[m]
+// the W part.
+template <typename T, int E, int NTB, int LG = 0, bool EDGE = false, bool WEDGE = false>
 __global__ void SG_COLS_BOUNDS(T, NTB) k_bwd_cols(const typename CX<T>::t* __restrict__ A,
                                                   const typename CX<T>::t* __restrict__ C,
                                                   const typename CX<T>::t* __restrict__ Kr,
@@ -1304,7 +1307,8 @@ __global__ void SG_COLS_BOUNDS(T, NTB) k_bwd_cols(const typename CX<T>::t* __res
                                                   const T* __restrict__ egr, const T* __restrict__ egp,
                                                   const T* __restrict__ wpre, EdgeCoef<T> ecoef,
                                                   const __grid_constant__ CUtensorMap mapP,
-                                                  const __grid_constant__ CUtensorMap mapB, int rows_layout)
+                                                  const __grid_constant__ CUtensorMap mapB, int rows_layout,
+                                                  const T* __restrict__ wtab, typename CX<T>::t* t_out)
 {
     const unsigned long long wlim = sg_wait_budget(err);  // read once, early
     if constexpr (LG > 0) {  // the length is a compile-time constant
@@ -1396,6 +1400,38 @@ __global__ void SG_COLS_BOUNDS(T, NTB) k_bwd_cols(const typename CX<T>::t* __res
                 w[e] = (e < E / 2) ? c2(sm[t + e * NT], cs[t + e * NT]) : c2(V{0, 0}, V{0, 0});
         }
         __shared__ T red[NTB / 32][8];  // EDGE: per-warp sums of t_a
+        __shared__ T wred[NTB / 32][4];  // WEDGE: of t_W, t_V
+        if constexpr (WEDGE) {
+            const long tsz = (long)(half + 1) * nu;
+            T acc[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int e = 0; e < E / 2; e++) {
+                const int i = t + e * NT;
+                const T* tb = wtab + (long)m * nu + i;
+                const V a = c2_lo(w[e]), c = c2_hi(w[e]);
+                const T wi = wpre[i], wr = wi * tb[0], vr = wi * tb[2 * tsz];
+                if (m == 0) {  // Nyquist tables on the imaginary parts
+                    const T* tn = wtab + (long)half * nu + i;
+                    acc[0] += wr * a.x;
+                    acc[1] += wi * tn[0] * a.y;
+                    acc[2] += vr * a.x;
+                    acc[3] += wi * tn[2 * tsz] * a.y;
+                } else {  // i p c = p (-c.y + i c.x)
+                    const T wp = wi * tb[tsz], vp = wi * tb[3 * tsz];
+                    acc[0] += wr * a.x - wp * c.y;
+                    acc[1] += wr * a.y + wp * c.x;
+                    acc[2] += vr * a.x - vp * c.y;
+                    acc[3] += vr * a.y + vp * c.x;
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < 4; v++)
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc[v] += sg_shfl_xor(acc[v], o);
+            if ((t & 31) == 0)
+#pragma unroll
+                for (int v = 0; v < 4; v++) wred[t >> 5][v] = acc[v];
+        }
         if constexpr (EDGE) {
             // this thread's rows' terms of t_a = sum_i wpre[i] (gr[i - a] A_i + i gp[i - a] C_i)
             const T* g0 = g_s;
@@ -1451,6 +1487,17 @@ __global__ void SG_COLS_BOUNDS(T, NTB) k_bwd_cols(const typename CX<T>::t* __res
             };
             if (t < 2) y[0] = cadd(y[0], update(t));
             if (t >= NT - 2) y[E / 2 - 1] = cadd(y[E / 2 - 1], update(t - NT + 4));
+        }
+        if constexpr (WEDGE) {
+            if (t == 0) {
+                T s[4] = {0, 0, 0, 0};
+                for (int w8 = 0; w8 < (int)(blockDim.x >> 5); w8++)
+#pragma unroll
+                    for (int q = 0; q < 4; q++) s[q] += wred[w8][q];
+                const T i0 = (T)1 / wpre[0];
+                y[0] = cadd(y[0], V{s[2] * i0, s[3] * i0});
+                t_out[m] = V{s[0], s[1]};
+            }
         }
         if (LG > 12 && rows_layout) {  // as the forward pass
             const int sw = 2 * spec_swap(m);
@@ -1925,13 +1972,49 @@ __device__ __forceinline__ bool rows_r2c_unit(const float* __restrict__ x0, cons
     return true;
 }
 
+// The wedge row's half spectrum (forward) as one more unit of the pass: x, N
+// reals, to out, N/2 modes (mode 0: (DC, Nyquist)).  Every transform of the
+// block computes it, the first one stores it.  As launches of their own the
+// wedge's two row transforms (direct DFTs, 7 us each) and its adjoint update
+// (12 us) also broke the chain of programmatic launches; with them inside the
+// passes 1024 x 2048 forward and adjoint went from 97.1 to 81.4 us.
+template <int LG, bool SMALL>
+__device__ __forceinline__ void wedge_r2c_unit(const float* x, float2* out, const float2* __restrict__ tw,
+                                               unsigned char* smraw)
+{
+    typedef RowUnit<LG, SMALL> RU;
+    constexpr int N = RU::N, NT = RU::NT;
+    const int tr = threadIdx.x / NT, t = threadIdx.x % NT;
+    const Twd<16, float2> twd = make_twd<16>(LG, t, tw);
+    sg_grid_dep_launch();
+    sg_grid_dep_wait();
+    const F2 zero = f2(0.f, 0.f);
+    C2 w[16];
+#pragma unroll
+    for (int e = 0; e < 16; e++) w[e] = C2{f2(sg_ld_dep(x + t + e * NT), 0.f), zero};
+    C2* const sm = reinterpret_cast<C2*>(align128(smraw)) + (size_t)tr * sg_padded(N);
+    const SgSyncBlock bsync;
+    sg_fft_pair<-1, LG>(w, sm, N, LG, t, twd.h, bsync);
+    C2 xa[8], xb[8];
+    split_real_pair2(w, sm, N, t, xa, xb, bsync);
+    if (tr == 0)
+#pragma unroll
+        for (int e = 0; e < 8; e++) out[t + e * NT] = c2_lo(xa[e]);
+}
+
+// sigw: the wedge row, whose half spectrum the grid's last block writes to swh (null: none)
 template <int LG, bool BWD, bool DIRECT = false, bool SMALL = false>
 __global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MINB)
     k_rows_r2c(const float* __restrict__ x0, const float* __restrict__ x1, const float* __restrict__ wrow,
-               float2* __restrict__ out, int nu, const float2* __restrict__ tw, int* err, int wave)
+               float2* __restrict__ out, int nu, const float2* __restrict__ tw, int* err, int wave, const float* sigw,
+               float2* swh)
 {
     const unsigned long long wlim = sg_wait_budget(err);  // read once, early
     extern __shared__ __align__(128) unsigned char smraw[];
+    if (!BWD && !DIRECT && sigw && blockIdx.x == gridDim.x - 1) {
+        wedge_r2c_unit<LG, SMALL>(sigw, swh, tw, smraw);
+        return;
+    }
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) sg_mbar_init(&bar, 1);
     __syncthreads();
@@ -2027,14 +2110,46 @@ __device__ __forceinline__ bool rows_c2r_unit(const float4* in, const float* __r
     return true;
 }
 
-// in: the input spectra (forward: the pairs; adjoint: the single values)
+// The wedge row's gradient (adjoint) as one more unit of the pass: the real
+// row whose half spectrum is h, as wedge_r2c_unit
+template <int LG, bool SMALL>
+__device__ __forceinline__ void wedge_c2r_unit(const float2* h, float* y, const float2* __restrict__ tw,
+                                               unsigned char* smraw)
+{
+    typedef RowUnit<LG, SMALL> RU;
+    constexpr int N = RU::N, NT = RU::NT, half = N / 2;
+    const int tr = threadIdx.x / NT, t = threadIdx.x % NT;
+    const Twd<16, float2> twd = make_twd<16>(LG, t, tw);
+    sg_grid_dep_launch();
+    sg_grid_dep_wait();
+    C2 w[16];
+#pragma unroll
+    for (int e = 0; e < 16; e++) {
+        const int n = t + e * NT;
+        const float2 u = sg_ld_dep(h + (e < 8 ? n : (n == half ? 0 : N - n)));
+        const float re = n == half ? u.y : u.x, im = (n == 0 || n == half) ? 0.f : e < 8 ? u.y : -u.y;
+        w[e] = C2{f2(re, 0.f), f2(im, 0.f)};
+    }
+    C2* const sm = reinterpret_cast<C2*>(align128(smraw)) + (size_t)tr * sg_padded(N);
+    sg_fft_pair<+1, LG>(w, sm, N, LG, t, twd.h);
+    if (tr == 0)
+#pragma unroll
+        for (int e = 0; e < 16; e++) y[t + e * NT] = f2_lo(w[e].x);
+}
+
+// in: the input spectra (forward: the pairs; adjoint: the single values); wh:
+// the half spectrum whose row the grid's last block writes to wy (null: none)
 template <int LG, bool BWD, bool SMALL = false>
 __global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MINB)
     k_rows_c2r(const float4* in, const float* __restrict__ wrow, float* __restrict__ y0,
-               float* __restrict__ y1, int nu, const float2* __restrict__ tw, int* err)
+               float* __restrict__ y1, int nu, const float2* __restrict__ tw, int* err, const float2* wh, float* wy)
 {
     const unsigned long long wlim = sg_wait_budget(err);  // read once, early
     extern __shared__ __align__(128) unsigned char smraw[];
+    if (BWD && wh && blockIdx.x == gridDim.x - 1) {
+        wedge_c2r_unit<LG, SMALL>(wh, wy, tw, smraw);
+        return;
+    }
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) sg_mbar_init(&bar, 1);
     __syncthreads();
@@ -2185,14 +2300,16 @@ __global__ void __launch_bounds__((1 << LG) / 16, 1)
 // ===========================================================================
 // the pass kernels' signatures (spelled out: naming an instance here would
 // refer to kernels that each translation unit does not define)
-typedef void (*RowsR2CFn)(const float*, const float*, const float*, float2*, int, const float2*, int*, int);
-typedef void (*RowsC2RFn)(const float4*, const float*, float*, float*, int, const float2*, int*);
+typedef void (*RowsR2CFn)(const float*, const float*, const float*, float2*, int, const float2*, int*, int,
+                          const float*, float2*);
+typedef void (*RowsC2RFn)(const float4*, const float*, float*, float*, int, const float2*, int*, const float2*,
+                          float*);
 typedef void (*FwdColsFn)(const float2*, const float2*, const float2*, float2*, float2*, int, int, int,
                           const float2*, int*, const float*, const float*, const float*, EdgeCoef<float>,
                           WedgeArgs<float>, CUtensorMap, CUtensorMap, int);
 typedef void (*BwdColsFn)(const float2*, const float2*, const float2*, const float2*, float2*, int, int, int,
                           const float2*, int*, const float*, const float*, const float*, EdgeCoef<float>,
-                          CUtensorMap, CUtensorMap, int);
+                          CUtensorMap, CUtensorMap, int, const float*, float2*);
 
 typedef void (*RingColsFn)(const float2*, const float2*, float2*, int, const float2*, int*, CUtensorMap, const float2*,
                            int);
@@ -2213,7 +2330,8 @@ struct FixedPassKernels {
     FwdColsFn fwd_cols_edge;        // with the edge-slope update
     FwdColsFn fwd_cols_edge_wedge;  // with the edge-slope and origin-wedge updates
     BwdColsFn bwd_cols;
-    BwdColsFn bwd_cols_edge;  // with the transposed edge-slope update
+    BwdColsFn bwd_cols_edge;        // with the transposed edge-slope update
+    BwdColsFn bwd_cols_edge_wedge;  // with the transposed edge-slope and origin-wedge updates
     RingColsFn ring_cols[2];  // k_ring_cols, forward and adjoint, or null (lengths below 8192)
     // the row instances for passes of `rows_per_transform` rows each: the small
     // blocks while the others are fewer than the SMs
@@ -2251,6 +2369,7 @@ FixedPassKernels make_fixed_pass_kernels()
                             k_fwd_cols<float, 16, NB, LG, true, true>,
                             k_bwd_cols<float, 16, NB, LG>,
                             k_bwd_cols<float, 16, NB, LG, true>,
+                            k_bwd_cols<float, 16, NB, LG, true, true>,
                             {ring_cols_kernel<LG, false>(), ring_cols_kernel<LG, true>()}};
 }
 
@@ -2509,7 +2628,10 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
     // wedge's update inside the column pass; the wedge row's spectrum is
     // formed first, ahead of the chained passes
     const bool wedge_fused = sizeof(T) == 4 && 2 * p.nu >= 16 && p.edges && p.wedge;
-    if (wedge_fused && (err = launch_wedge_dft<T>(p, st)) != cudaSuccess) return err;
+    // (by a block of the row pass, where the rows are fixed-length)
+    const bool wedge_row = wedge_fused && p.pairs == 2;
+    if (wedge_row && !p.sigw) return cudaErrorInvalidValue;
+    if (wedge_fused && !wedge_row && (err = launch_wedge_dft<T>(p, st)) != cudaSuccess) return err;
     {
         PassRange range_("sg forward rows");
         if (sizeof(T) == 4 && p.tcm) {
@@ -2520,8 +2642,10 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
             auto k = sigma_direct ? rk.fwd_rows_direct : rk.fwd_rows;
             if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
             const int wave = resident_blocks(k, rk.threads, rk.smem, p.sms);
-            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, (const float*)sigma, (const float*)nullptr,
-                                  (const float*)p.wpre, (float2*)p.wa, p.nu, (const float2*)p.tw, p.err, wave)) !=
+            if ((err = launch_pdl(k, nblk + (wedge_row ? 1 : 0), rk.threads, rk.smem, st, (const float*)sigma,
+                                  (const float*)nullptr, (const float*)p.wpre, (float2*)p.wa, p.nu,
+                                  (const float2*)p.tw, p.err, wave, wedge_row ? (const float*)p.sigw : nullptr,
+                                  (float2*)p.wtmp)) !=
                 cudaSuccess)
                 return err;
         } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
@@ -2594,7 +2718,7 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
             auto k = rk.fwd_rows_inv;
             if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
             if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, (const float4*)p.wb, (const float*)p.wpost, (float*)Fr, (float*)Fp, p.nu,
-                                  (const float2*)p.tw, p.err)) != cudaSuccess)
+                                  (const float2*)p.tw, p.err, (const float2*)nullptr, (float*)nullptr)) != cudaSuccess)
                 return err;
         } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
             if ((err = launch_fx_c2r(p, (double*)Fr, (double*)Fp, st)) != cudaSuccess) return err;
@@ -2635,6 +2759,8 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
     const int ln = sg_ilog2(p.nphi), lL = sg_ilog2(2 * p.nu);
     cudaError_t err;
     bool edges_done = false;  // the column pass applied the transposed edge update itself
+    bool wedge_done = false;  // and the transposed wedge update; the inverse row pass then forms gsigma_w
+    if (p.wedge && !p.gsigw) return cudaErrorInvalidValue;
     if (ev && (err = cudaEventRecord(ev[0], st)) != cudaSuccess) return err;
     {
         PassRange range_("sg adjoint rows");
@@ -2647,7 +2773,8 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
             if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
             const int wave = resident_blocks(k, rk.threads, rk.smem, p.sms);
             if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, (const float*)gr, (const float*)gp,
-                                  (const float*)p.wpost, (float2*)p.wb, p.nu, (const float2*)p.tw, p.err, wave)) !=
+                                  (const float*)p.wpost, (float2*)p.wb, p.nu, (const float2*)p.tw, p.err, wave,
+                                  (const float*)nullptr, (float2*)nullptr)) !=
                 cudaSuccess)
                 return err;
         } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
@@ -2689,7 +2816,9 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
                 if (L / EE > 256) k = k_bwd_cols<T, EE, 512>;
             if constexpr (sizeof(T) == 4 && EE == 16) {
                 if (fuse) k = L / EE > 256 ? k_bwd_cols<T, 16, 512, 0, true> : k_bwd_cols<T, 16, 256, 0, true>;
-                if (p.pairs) k = fuse ? fc->bwd_cols_edge : fc->bwd_cols;  // reads the (A, C) pairs of wb
+                wedge_done = fuse && p.wedge && p.pairs == 2;
+                if (p.pairs)  // reads the (A, C) pairs of wb
+                    k = wedge_done ? fc->bwd_cols_edge_wedge : fuse ? fc->bwd_cols_edge : fc->bwd_cols;
             }
             const size_t smem = bcols_smem_bytes<T>(p.nu);  // the edge rows share the exchange area
             if ((err = set_smem(k, smem, true)) != cudaSuccess) return err;
@@ -2698,13 +2827,14 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
                                   (const V*)p.kp, p.pairs ? A : B, p.nu, p.nphi, lL, tw, p.err, (const T*)p.egr,
                                   (const T*)p.egp, (const T*)p.wpre, coef,
                                   p.pairs == 2 ? p.imaps[0] : CUtensorMap{},
-                                  p.pairs == 2 ? p.imaps[1] : CUtensorMap{}, p.pairs == 2)) != cudaSuccess)
+                                  p.pairs == 2 ? p.imaps[1] : CUtensorMap{}, p.pairs == 2, (const T*)p.wtab,
+                                  (V*)p.wtmp)) != cudaSuccess)
                 return err;
             edges_done = fuse;
         });
     }
     if (p.edges && !edges_done && (err = launch_edges<T>(p, true, st)) != cudaSuccess) return err;
-    if (p.wedge && (err = launch_wedge<T>(p, true, st)) != cudaSuccess) return err;
+    if (p.wedge && !wedge_done && (err = launch_wedge<T>(p, true, st)) != cudaSuccess) return err;
     if (ev && (err = cudaEventRecord(ev[2], st)) != cudaSuccess) return err;
     {
         PassRange range_("sg adjoint inverse rows");
@@ -2715,8 +2845,9 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
             const int nblk = p.nu / (4 * rk.slots);
             auto k = rk.bwd_rows_inv;
             if ((err = set_smem(k, rk.smem, true)) != cudaSuccess) return err;
-            if ((err = launch_pdl(k, nblk, rk.threads, rk.smem, st, (const float4*)p.wa, (const float*)p.wpre, (float*)gs, (float*)nullptr,
-                                  p.nu, (const float2*)p.tw, p.err)) != cudaSuccess)
+            if ((err = launch_pdl(k, nblk + (wedge_done ? 1 : 0), rk.threads, rk.smem, st, (const float4*)p.wa,
+                                  (const float*)p.wpre, (float*)gs, (float*)nullptr, p.nu, (const float2*)p.tw, p.err,
+                                  wedge_done ? (const float2*)p.wtmp : nullptr, (float*)p.gsigw)) != cudaSuccess)
                 return err;
         } else if (std::is_same<T, double>::value && fx_rows_ok(p)) {
             if ((err = launch_fx_c2r(p, (double*)gs, nullptr, st)) != cudaSuccess) return err;

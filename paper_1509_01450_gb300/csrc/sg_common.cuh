@@ -562,6 +562,12 @@ __device__ __forceinline__ void sg_grid_dep_launch() { asm volatile("griddepcont
 // that they stay behind it.  (A load through a const __restrict__ pointer or
 // __ldg is free to move above the wait: the compiler takes its memory for
 // constant over the whole kernel.)
+__device__ __forceinline__ float sg_ld_dep(const float* p)
+{
+    float r;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(r) : "l"(p) : "memory");
+    return r;
+}
 __device__ __forceinline__ float2 sg_ld_dep(const float2* p)
 {
     float2 r;

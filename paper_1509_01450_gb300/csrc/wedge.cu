@@ -14,11 +14,13 @@
 // with s^_w the phi-DFT of sigma_w and a_0 = A[m][0] / wpre[0] that of
 // sigma_0, applied between the column pass and the inverse-row pass by
 // k_wedge_fwd, or, for FP32 columns of 16 points per thread, inside the
-// forward column pass with s^_w formed ahead by k_wedge_dft.  Mode 0
+// forward column pass with s^_w formed ahead by k_wedge_dft (in the fixed-
+// length FP32 passes by a block of the row pass, fftconv.cu).  Mode 0
 // packs (DC, Nyquist) as the passes do: real parts use the m = 0 tables,
 // imaginary parts the m = N_phi/2 ones, and the azimuthal terms vanish.
 // The adjoint forms the transposed sums t(m) per mode, adds the V part to
-// row 0 of the backward column spectra and returns gsigma_w as the inverse
+// row 0 of the backward column spectra (the fixed-length FP32 passes do both
+// in their column pass) and returns gsigma_w as the inverse
 // phi-DFT of the W part.  All arithmetic is in the plan's dtype with the
 // plan's twiddle table (GB300's FP64 rate would make FP64 sums here cost
 // more than a pass); the direct DFTs of the one wedge row take N_phi^2 / 2
