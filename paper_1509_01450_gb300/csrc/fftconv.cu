@@ -1863,6 +1863,41 @@ __host__ __device__ __forceinline__ size_t rows_unit_smem_bytes()
     return RowUnit<LG, SMALL>::SMEM;
 }
 
+// One transform's part of the row R2C pass, from its four real rows (rp, rq,
+// rr, rs), z1 = rp + i rq, z2 = rr + i rs, times the weights wt, to the units
+// of rows i0 on; sm: its exchange area.  The syncs are block barriers: rsync
+// once the rows are read, xsync in the transform, ssync in the split (its
+// second call finds the area free).
+template <int LG, bool BWD, typename RSync, typename XSync, typename SSync>
+__device__ __forceinline__ void rows_r2c_math(const float* rp, const float* rq, const float* rr, const float* rs,
+                                              const float (&wt)[4], C2* sm, const Twd<16, float2>& twd,
+                                              float2* __restrict__ out, int i0, int nu, int t, int* err,
+                                              const RSync& rsync, const XSync& xsync, const SSync& ssync)
+{
+    constexpr int N = 1 << LG, NT = N / 16, RPT = BWD ? 2 : 4;
+    const F2 wx = f2(wt[0], wt[2]), wy = f2(wt[1], wt[3]);
+    C2 w[16];
+#pragma unroll
+    for (int e = 0; e < 16; e++) {
+        const int n = t + e * NT;
+        w[e] = C2{f2(rp[n], rr[n]) * wx, f2(rq[n], rs[n]) * wy};
+    }
+    rsync();  // every transform has read its rows
+    sg_fft_pair<-1, LG>(w, sm, N, LG, t, twd.h, xsync);
+    C2 xa[8], xb[8];
+    split_real_pair2(w, sm, N, t, xa, xb, ssync);
+    // forward: A of rows i0..i0+3; adjoint: {A, C} of rows i0, i0+1: one unit a mode
+    const uint64_t keep = sg_policy_evict_last();  // the column pass reads the spectra from L2
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        const size_t unit = (size_t)(i0 / RPT) * (N / 2) + t + e * NT;
+        float* q = reinterpret_cast<float*>(out) + 8 * unit;
+        SG_IF_OK(sg_in((long long)unit, 1, (long long)(N / 2) * (nu / RPT)), err, 103)
+        sg_st256_hint(q, make_float4(f2_lo(xa[e].x), f2_lo(xa[e].y), f2_lo(xb[e].x), f2_lo(xb[e].y)),
+                      make_float4(f2_hi(xa[e].x), f2_hi(xa[e].y), f2_hi(xb[e].x), f2_hi(xb[e].y)), keep);
+    }
+}
+
 // DIRECT (forward only): sigma is memory the GPU reaches only by plain loads
 // (pinned host memory), read straight into registers without bulk copies
 // One unit of the row R2C pass: rows u R .. u R + R - 1 (the pass kernel
@@ -1946,29 +1981,9 @@ __device__ __forceinline__ bool rows_r2c_unit(const float* __restrict__ x0, cons
             rs = rp + 3 * N;
         }
     }
-    const F2 wx = f2(wt[0], wt[2]), wy = f2(wt[1], wt[3]);
-    C2 w[16];
-#pragma unroll
-    for (int e = 0; e < 16; e++) {
-        const int n = t + e * NT;
-        w[e] = C2{f2(rp[n], rr[n]) * wx, f2(rq[n], rs[n]) * wy};
-    }
-    __syncthreads();  // every transform has read its rows: the area holds the exchange areas
-    C2* const sm = reinterpret_cast<C2*>(area) + (size_t)tr * sg_padded(N);
     const SgSyncBlock bsync;
-    sg_fft_pair<-1, LG>(w, sm, N, LG, t, twd.h, bsync);
-    C2 xa[8], xb[8];
-    split_real_pair2(w, sm, N, t, xa, xb, bsync);
-    // forward: A of rows i0..i0+3; adjoint: {A, C} of rows i0, i0+1: one unit a mode
-    const uint64_t keep = sg_policy_evict_last();  // the column pass reads the spectra from L2
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-        const size_t unit = (size_t)(i0 / RPT) * (N / 2) + t + e * NT;
-        float* q = reinterpret_cast<float*>(out) + 8 * unit;
-        SG_IF_OK(sg_in((long long)unit, 1, (long long)(N / 2) * (nu / RPT)), err, 103)
-        sg_st256_hint(q, make_float4(f2_lo(xa[e].x), f2_lo(xa[e].y), f2_lo(xb[e].x), f2_lo(xb[e].y)),
-                      make_float4(f2_hi(xa[e].x), f2_hi(xa[e].y), f2_hi(xb[e].x), f2_hi(xb[e].y)), keep);
-    }
+    rows_r2c_math<LG, BWD>(rp, rq, rr, rs, wt, reinterpret_cast<C2*>(area) + (size_t)tr * sg_padded(N), twd, out, i0, nu,
+                           t, err, bsync, bsync, bsync);  // the exchange areas lie over the rows
     return true;
 }
 
@@ -2022,45 +2037,16 @@ __global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MI
     rows_r2c_unit<LG, BWD, DIRECT, true, SMALL>(x0, x1, wrow, out, nu, tw, err, blockIdx.x, wave, smraw, bar, 0, wlim);
 }
 
-// One unit of the row C2R pass (rows u R .. u R + R - 1), shared like
-// rows_r2c_unit; map: the tensor map in kernel-parameter or global memory.
-template <int LG, bool BWD, bool PDL, bool SMALL = false>
-__device__ __forceinline__ bool rows_c2r_unit(const float4* in, const float* __restrict__ wrow,
-                                              float* __restrict__ y0, float* __restrict__ y1, int nu,
-                                              const float2* __restrict__ tw, int* err, int u, unsigned char* smraw,
-                                              uint64_t& bar, uint32_t phase, unsigned long long wlim,
-                                              bool* landed = nullptr)
+// One transform's part of the row C2R pass, from its modes' units at S4 to the
+// rows i0 on, times the weights wt; sm: its exchange area; rsync, xsync as in
+// rows_r2c_math (the transform's last barrier finds the area free).
+template <int LG, bool BWD, typename RSync, typename XSync>
+__device__ __forceinline__ void rows_c2r_math(const float4* S4, const float (&wt)[4], C2* sm,
+                                              const Twd<16, float2>& twd, float* __restrict__ y0,
+                                              float* __restrict__ y1, int i0, int nu, int t, int* err,
+                                              const RSync& rsync, const XSync& xsync)
 {
-    typedef RowUnit<LG, SMALL> RU;
-    constexpr int N = RU::N, NT = RU::NT, TPG = RU::TPG, half = N / 2;
-    constexpr int RPT = BWD ? 4 : 2;  // rows per transform
-    constexpr int R = RPT * TPG;      // rows per block
-    unsigned char* const area = align128(smraw);
-    const int tr = threadIdx.x / NT, t = threadIdx.x % NT;
-    const int i0 = u * R + tr * RPT;
-    const Twd<16, float2> twd = make_twd<16>(LG, t, tw);
-    // the output rows' weights: forward (w_i0, w_i0, w_i0+1, w_i0+1), adjoint w_i0..i0+3
-    float wt[4] = {0.f, 0.f, 0.f, 0.f};
-    const bool rows_ok = i0 + (BWD ? 4 : 2) <= nu;
-    (void)rows_ok;  // read by the checked build only
-    SG_IF_OK(rows_ok, err, 201) {
-#pragma unroll
-        for (int r = 0; r < 4; r++) wt[r] = __ldg(&wrow[i0 + (BWD ? r : r / 2)]);
-    }
-    if constexpr (PDL) {
-        sg_grid_dep_launch();
-        sg_grid_dep_wait();  // the spectra are the previous pass's results
-    }
-    if (threadIdx.x == 0) {
-        // transform j's rows land at j N x 16 bytes, mode n of them at 32 n
-        constexpr uint32_t bytes = (uint32_t)(TPG * half * 32);
-        sg_mbar_expect_tx(&bar, bytes);
-        const long long unit = (long long)u * TPG * half;
-        SG_IF_OK(sg_in(unit, TPG * half, (long long)half * (nu / RPT)) && sg_smem_in(smraw, area, bytes), err, 202)
-        sg_bulk_g2s_hint(area, in + 2 * unit, bytes, &bar, sg_policy_evict_first());  // consumed here
-    }
-    if (__syncthreads_or(!sg_mbar_wait_bounded(&bar, phase, err, 1, wlim, landed))) return false;  // inputs never arrived
-    const float4* const S4 = reinterpret_cast<const float4*>(area) + (size_t)tr * N;  // this transform's modes
+    constexpr int N = 1 << LG, NT = N / 16, half = N / 2;
     // Z of both lanes at frequency n.  Each mode holds two 16-byte halves u0,
     // u1 (forward: {B, C} of rows i0, i0+1; adjoint: {S_i0, S_i0+1}, {S_i0+2,
     // S_i0+3}), swapped for modes with bit 2 set.
@@ -2083,8 +2069,8 @@ __device__ __forceinline__ bool rows_c2r_unit(const float4* in, const float* __r
         else
             w[e] = C2{f2(u0.x + u0.w, u1.x + u1.w), f2(u0.z - u0.y, u1.z - u1.y)};
     }
-    __syncthreads();  // the exchange areas lie over the other transforms' stages
-    sg_fft_pair<+1, LG>(w, reinterpret_cast<C2*>(area) + (size_t)tr * sg_padded(N), N, LG, t, twd.h);
+    rsync();  // every transform has read its modes
+    sg_fft_pair<+1, LG>(w, sm, N, LG, t, twd.h, xsync);
     // the four output rows: forward (F_r, F_phi) of i0, then of i0+1;
     // adjoint gsigma of i0 .. i0+3; values Re, Im of the low, then high lanes
     float* o[4];
@@ -2097,7 +2083,7 @@ __device__ __forceinline__ bool rows_c2r_unit(const float4* in, const float* __r
         o[2] = y0 + (size_t)(i0 + 1) * N;
         o[3] = y1 + (size_t)(i0 + 1) * N;
     }
-    SG_IF_OK(rows_ok, err, 203) {
+    SG_IF_OK(i0 + (BWD ? 4 : 2) <= nu, err, 203) {
 #pragma unroll
         for (int e = 0; e < 16; e++) {
             const int n = t + e * NT;
@@ -2107,6 +2093,48 @@ __device__ __forceinline__ bool rows_c2r_unit(const float4* in, const float* __r
             o[3][n] = f2_hi(w[e].y) * wt[3];
         }
     }
+}
+
+// One unit of the row C2R pass (rows u R .. u R + R - 1), shared like
+// rows_r2c_unit; map: the tensor map in kernel-parameter or global memory.
+template <int LG, bool BWD, bool PDL, bool SMALL = false>
+__device__ __forceinline__ bool rows_c2r_unit(const float4* in, const float* __restrict__ wrow,
+                                              float* __restrict__ y0, float* __restrict__ y1, int nu,
+                                              const float2* __restrict__ tw, int* err, int u, unsigned char* smraw,
+                                              uint64_t& bar, uint32_t phase, unsigned long long wlim,
+                                              bool* landed = nullptr)
+{
+    typedef RowUnit<LG, SMALL> RU;
+    constexpr int N = RU::N, NT = RU::NT, TPG = RU::TPG, half = N / 2;
+    constexpr int RPT = BWD ? 4 : 2;  // rows per transform
+    constexpr int R = RPT * TPG;      // rows per block
+    unsigned char* const area = align128(smraw);
+    const int tr = threadIdx.x / NT, t = threadIdx.x % NT;
+    const int i0 = u * R + tr * RPT;
+    const Twd<16, float2> twd = make_twd<16>(LG, t, tw);
+    // the output rows' weights: forward (w_i0, w_i0, w_i0+1, w_i0+1), adjoint w_i0..i0+3
+    float wt[4] = {0.f, 0.f, 0.f, 0.f};
+    SG_IF_OK(i0 + (BWD ? 4 : 2) <= nu, err, 201) {
+#pragma unroll
+        for (int r = 0; r < 4; r++) wt[r] = __ldg(&wrow[i0 + (BWD ? r : r / 2)]);
+    }
+    if constexpr (PDL) {
+        sg_grid_dep_launch();
+        sg_grid_dep_wait();  // the spectra are the previous pass's results
+    }
+    if (threadIdx.x == 0) {
+        // transform j's rows land at j N x 16 bytes, mode n of them at 32 n
+        constexpr uint32_t bytes = (uint32_t)(TPG * half * 32);
+        sg_mbar_expect_tx(&bar, bytes);
+        const long long unit = (long long)u * TPG * half;
+        SG_IF_OK(sg_in(unit, TPG * half, (long long)half * (nu / RPT)) && sg_smem_in(smraw, area, bytes), err, 202)
+        sg_bulk_g2s_hint(area, in + 2 * unit, bytes, &bar, sg_policy_evict_first());  // consumed here
+    }
+    if (__syncthreads_or(!sg_mbar_wait_bounded(&bar, phase, err, 1, wlim, landed))) return false;  // inputs never arrived
+    const float4* const S4 = reinterpret_cast<const float4*>(area) + (size_t)tr * N;  // this transform's modes
+    const SgSyncBlock bsync;
+    rows_c2r_math<LG, BWD>(S4, wt, reinterpret_cast<C2*>(area) + (size_t)tr * sg_padded(N), twd, y0, y1, i0, nu, t, err,
+                           bsync, bsync);  // the exchange areas lie over the other transforms' stages
     return true;
 }
 
@@ -2156,6 +2184,147 @@ __global__ void __launch_bounds__(RowUnit<LG, SMALL>::GT, RowUnit<LG, SMALL>::MI
     rows_c2r_unit<LG, BWD, true, SMALL>(in, wrow, y0, y1, nu, tw, err, blockIdx.x, smraw, bar, 0, wlim);
 }
 
+// A block barrier whose nth call also runs fn on thread 0, once every thread
+// has arrived and its shared-memory accesses come before fn's copies.
+template <typename F>
+struct SgSyncThen {
+    F fn;
+    mutable int left;
+    __device__ __forceinline__ explicit SgSyncThen(F f, int nth = 1) : fn(f), left(nth) {}
+    __device__ __forceinline__ void operator()() const
+    {
+        left--;
+        if (left == 0) sg_fence_proxy_async();
+        __syncthreads();
+        if (left == 0 && threadIdx.x == 0) fn();
+    }
+};
+
+// ===========================================================================
+// The row passes for 8192 points, whose area leaves room for one block per SM:
+// nothing else hides a block's copies there, so the blocks are persistent and
+// a 64 KB buffer precedes the exchange area.  A unit's 128 KB of input lie
+// over both: the first half of the next unit's arrives in the buffer while
+// this unit transforms, the second half in the exchange area from the
+// transform's last exchange on (while its results are stored).
+// 4096 x 8192, one block per unit -> persistent, us: R2C 88.7 -> 81.7, C2R
+// 159.7 -> 141.3; adjoint R2C 160.6 -> 153.8, C2R 88.0 -> 73.7.
+// ===========================================================================
+template <int LG>
+__host__ __device__ __forceinline__ size_t ring_rows_smem_bytes()
+{
+    return ((size_t)8 << LG) + (size_t)sg_padded(1 << LG) * sizeof(C2) + 128;  // + the alignment slack
+}
+
+template <int LG, bool BWD>
+__global__ void __launch_bounds__((1 << LG) / 16, 1)
+    k_ring_rows_r2c(const float* __restrict__ x0, const float* __restrict__ x1, const float* __restrict__ wrow,
+                    float2* __restrict__ out, int nu, const float2* __restrict__ tw, int* err)
+{
+    constexpr int N = 1 << LG, RPT = BWD ? 2 : 4;
+    constexpr uint32_t hb = 2 * N * 4;  // bytes of two rows: half a unit's input, the buffer's size
+    const unsigned long long wlim = sg_wait_budget(err);  // read once, early
+    extern __shared__ __align__(128) unsigned char smraw[];
+    __shared__ __align__(8) uint64_t bar[2];  // the halves
+    unsigned char* const buf = align128(smraw);
+    const float* const in = reinterpret_cast<const float*>(buf);
+    C2* const sm = reinterpret_cast<C2*>(buf + hb);
+    const int t = threadIdx.x, units = nu / RPT;
+    if (t == 0) {
+        sg_mbar_init(&bar[0], 1);
+        sg_mbar_init(&bar[1], 1);
+    }
+    __syncthreads();
+    const Twd<16, float2> twd = make_twd<16>(LG, t, tw);
+    const uint64_t drop = sg_policy_evict_first();
+    // thread 0, with the half free: forward rows i0, i0 + 1 | i0 + 2, i0 + 3 of sigma; adjoint gF_r | gF_phi
+    const auto issue = [&](int u, int h) {
+        sg_mbar_expect_tx(&bar[h], hb);
+        const float* const src = BWD ? (h ? x1 : x0) + (size_t)u * RPT * N : x0 + ((size_t)u * RPT + 2 * h) * N;
+        SG_IF_OK(u < units && sg_smem_in(smraw, buf + h * hb, hb), err, 105)
+        sg_bulk_g2s_hint(buf + h * hb, src, hb, &bar[h], drop);
+    };
+    sg_grid_dep_launch();
+    sg_grid_dep_wait();  // the inputs may come from the previous kernel on the stream
+    if (t == 0) {
+        issue(blockIdx.x, 0);
+        issue(blockIdx.x, 1);
+    }
+    uint32_t ph = 0;
+    for (int u = blockIdx.x; u < units; u += gridDim.x, ph ^= 1) {
+        const int i0 = u * RPT, next = u + gridDim.x;
+        float wt[4];
+#pragma unroll
+        for (int r = 0; r < 4; r++) wt[r] = __ldg(&wrow[i0 + (BWD ? r / 2 : r)]);
+        const bool in0 = sg_mbar_wait_bounded(&bar[0], ph, err, 1, wlim);
+        const bool in1 = sg_mbar_wait_bounded(&bar[1], ph, err, 1, wlim);
+        if (__syncthreads_or(!in0 || !in1)) return;  // the unit's input never arrived
+        const auto next0 = [&] {
+            if (next < units) issue(next, 0);
+        };
+        const auto next1 = [&] {
+            if (next < units) issue(next, 1);
+        };
+        const float *r1 = in + N, *r2 = in + 2 * N, *r3 = in + 3 * N;  // rows in the order they lie
+        rows_r2c_math<LG, BWD>(in, BWD ? r2 : r1, BWD ? r1 : r2, r3, wt, sm, twd, out, i0, nu, t, err,
+                               SgSyncThen<decltype(next0)>(next0), SgSyncBlock(),
+                               SgSyncThen<decltype(next1)>(next1, 2));
+    }
+}
+
+template <int LG, bool BWD>
+__global__ void __launch_bounds__((1 << LG) / 16, 1)
+    k_ring_rows_c2r(const float4* in, const float* __restrict__ wrow, float* __restrict__ y0,
+                    float* __restrict__ y1, int nu, const float2* __restrict__ tw, int* err)
+{
+    constexpr int N = 1 << LG, half = N / 2, RPT = BWD ? 4 : 2;
+    constexpr uint32_t hb = half / 2 * 32;  // bytes of half the modes, the buffer's size
+    constexpr int last = 1 + 2 * ((LG - 1) / 4);  // barriers of sg_fft_pair
+    const unsigned long long wlim = sg_wait_budget(err);  // read once, early
+    extern __shared__ __align__(128) unsigned char smraw[];
+    __shared__ __align__(8) uint64_t bar[2];  // the halves
+    unsigned char* const buf = align128(smraw);
+    C2* const sm = reinterpret_cast<C2*>(buf + hb);
+    const int t = threadIdx.x, units = nu / RPT;
+    if (t == 0) {
+        sg_mbar_init(&bar[0], 1);
+        sg_mbar_init(&bar[1], 1);
+    }
+    __syncthreads();
+    const Twd<16, float2> twd = make_twd<16>(LG, t, tw);
+    const uint64_t drop = sg_policy_evict_first();
+    // thread 0, with the half free: modes h N/4 .. (h + 1) N/4 - 1 of the unit
+    const auto issue = [&](int u, int h) {
+        sg_mbar_expect_tx(&bar[h], hb);
+        SG_IF_OK(u < units && sg_smem_in(smraw, buf + h * hb, hb), err, 204)
+        sg_bulk_g2s_hint(buf + h * hb, in + 2 * ((size_t)u * half + h * (half / 2)), hb, &bar[h], drop);
+    };
+    sg_grid_dep_launch();
+    sg_grid_dep_wait();  // the spectra are the previous pass's results
+    if (t == 0) {
+        issue(blockIdx.x, 0);
+        issue(blockIdx.x, 1);
+    }
+    uint32_t ph = 0;
+    for (int u = blockIdx.x; u < units; u += gridDim.x, ph ^= 1) {
+        const int i0 = u * RPT, next = u + gridDim.x;
+        float wt[4];
+#pragma unroll
+        for (int r = 0; r < 4; r++) wt[r] = __ldg(&wrow[i0 + (BWD ? r : r / 2)]);
+        const bool in0 = sg_mbar_wait_bounded(&bar[0], ph, err, 1, wlim);
+        const bool in1 = sg_mbar_wait_bounded(&bar[1], ph, err, 1, wlim);
+        if (__syncthreads_or(!in0 || !in1)) return;  // the unit's input never arrived
+        const auto next0 = [&] {
+            if (next < units) issue(next, 0);
+        };
+        const auto next1 = [&] {
+            if (next < units) issue(next, 1);
+        };
+        rows_c2r_math<LG, BWD>(reinterpret_cast<const float4*>(buf), wt, sm, twd, y0, y1, i0, nu, t, err,
+                               SgSyncThen<decltype(next0)>(next0), SgSyncThen<decltype(next1)>(next1, last));
+    }
+}
+
 // ===========================================================================
 // The column passes for 8192 points (N_u = 4096), whose exchange area leaves
 // room for one block per SM: nothing else hides a block's copies there, so the
@@ -2171,21 +2340,6 @@ __host__ __device__ __forceinline__ size_t ring_cols_smem_bytes(int nu)
 {
     return ring_cols_buffer(nu) + 2 * (size_t)(nu + 2) * sizeof(float2);
 }
-// a block barrier whose first call also runs fn on thread 0, once every
-// thread has arrived
-template <typename F>
-struct SgSyncThen {
-    F fn;
-    mutable bool done = false;
-    __device__ __forceinline__ explicit SgSyncThen(F f) : fn(f) {}
-    __device__ __forceinline__ void operator()() const
-    {
-        __syncthreads();
-        if (!done && threadIdx.x == 0) fn();
-        done = true;
-    }
-};
-
 template <int LG, bool BWD>
 __global__ void __launch_bounds__((1 << LG) / 16, 1)
     k_ring_cols(const float2* __restrict__ Kr, const float2* __restrict__ Kp, float2* __restrict__ out, int half,
@@ -2314,6 +2468,9 @@ typedef void (*BwdColsFn)(const float2*, const float2*, const float2*, const flo
 typedef void (*RingColsFn)(const float2*, const float2*, float2*, int, const float2*, int*, CUtensorMap, const float2*,
                            int);
 
+typedef void (*RingR2CFn)(const float*, const float*, const float*, float2*, int, const float2*, int*);
+typedef void (*RingC2RFn)(const float4*, const float*, float*, float*, int, const float2*, int*);
+
 struct FixedRowKernels {
     RowsR2CFn fwd_rows;         // k_rows_r2c, forward
     RowsR2CFn fwd_rows_direct;  // the same reading sigma from host memory the GPU can reach
@@ -2332,7 +2489,11 @@ struct FixedPassKernels {
     BwdColsFn bwd_cols;
     BwdColsFn bwd_cols_edge;        // with the transposed edge-slope update
     BwdColsFn bwd_cols_edge_wedge;  // with the transposed edge-slope and origin-wedge updates
-    RingColsFn ring_cols[2];  // k_ring_cols, forward and adjoint, or null (lengths below 8192)
+    // the persistent passes, forward and adjoint, or null (lengths below 8192)
+    RingColsFn ring_cols[2];
+    RingR2CFn ring_r2c[2];
+    RingC2RFn ring_c2r[2];
+    size_t ring_rows_smem;
     // the row instances for passes of `rows_per_transform` rows each: the small
     // blocks while the others are fewer than the SMs
     const FixedRowKernels& pick(int nu, int rows_per_transform, int sms) const
@@ -2350,27 +2511,28 @@ FixedRowKernels make_fixed_row_kernels()
                            k_rows_c2r<LG, true, SMALL>,        RU::SMEM,
                            RU::GT,                             RU::TPG};
 }
-template <int LG, bool BWD>
-RingColsFn ring_cols_kernel()
-{
-    if constexpr (LG > 12)
-        return k_ring_cols<LG, BWD>;
-    else
-        return nullptr;
-}
 template <int LG>
 FixedPassKernels make_fixed_pass_kernels()
 {
     constexpr int NB = (1 << LG) / 16 > 256 ? 512 : 256;
-    return FixedPassKernels{make_fixed_row_kernels<LG, false>(),
-                            make_fixed_row_kernels<LG, (LG < 12)>(),  // one transform fills a block from 4096 points on
-                            k_fwd_cols<float, 16, NB, LG>,
-                            k_fwd_cols<float, 16, NB, LG, true>,
-                            k_fwd_cols<float, 16, NB, LG, true, true>,
-                            k_bwd_cols<float, 16, NB, LG>,
-                            k_bwd_cols<float, 16, NB, LG, true>,
-                            k_bwd_cols<float, 16, NB, LG, true, true>,
-                            {ring_cols_kernel<LG, false>(), ring_cols_kernel<LG, true>()}};
+    FixedPassKernels k{make_fixed_row_kernels<LG, false>(),
+                       make_fixed_row_kernels<LG, (LG < 12)>(),  // one transform fills a block from 4096 points on
+                       k_fwd_cols<float, 16, NB, LG>,
+                       k_fwd_cols<float, 16, NB, LG, true>,
+                       k_fwd_cols<float, 16, NB, LG, true, true>,
+                       k_bwd_cols<float, 16, NB, LG>,
+                       k_bwd_cols<float, 16, NB, LG, true>,
+                       k_bwd_cols<float, 16, NB, LG, true, true>};
+    if constexpr (LG > 12) {
+        k.ring_cols[0] = k_ring_cols<LG, false>;
+        k.ring_cols[1] = k_ring_cols<LG, true>;
+        k.ring_r2c[0] = k_ring_rows_r2c<LG, false>;
+        k.ring_r2c[1] = k_ring_rows_r2c<LG, true>;
+        k.ring_c2r[0] = k_ring_rows_c2r<LG, false>;
+        k.ring_c2r[1] = k_ring_rows_c2r<LG, true>;
+        k.ring_rows_smem = ring_rows_smem_bytes<LG>();
+    }
+    return k;
 }
 
 // defined in fftconv_lg<LG>.cu
@@ -2594,6 +2756,31 @@ static bool ring_cols_fit(const PlanView& p, const FixedPassKernels* fc)
 {
     return p.pairs && !p.edges && fc->ring_cols[0] && p.nphi / 2 > p.sms;
 }
+// The persistent row passes, rows_per_unit rows each: not for at most one unit
+// per SM, which they would only delay, nor for the wedge's extra row.
+static bool ring_rows_fit(const PlanView& p, const FixedPassKernels* fr, int rows_per_unit, bool wedge)
+{
+    return fr->ring_rows_smem && !wedge && p.nu / rows_per_unit > p.sms;
+}
+static cudaError_t launch_ring_r2c(const PlanView& p, const FixedPassKernels* fr, bool adjoint, const float* x0,
+                                   const float* x1, cudaStream_t st)
+{
+    const RingR2CFn k = fr->ring_r2c[adjoint];
+    const cudaError_t err = set_smem(k, fr->ring_rows_smem, true);
+    if (err != cudaSuccess) return err;
+    return launch_pdl(k, p.sms, p.nphi / 16, fr->ring_rows_smem, st, x0, x1, (const float*)(adjoint ? p.wpost : p.wpre),
+                      (float2*)(adjoint ? p.wb : p.wa), p.nu, (const float2*)p.tw, p.err);
+}
+static cudaError_t launch_ring_c2r(const PlanView& p, const FixedPassKernels* fr, bool adjoint, float* y0, float* y1,
+                                   cudaStream_t st)
+{
+    const RingC2RFn k = fr->ring_c2r[adjoint];
+    const cudaError_t err = set_smem(k, fr->ring_rows_smem, true);
+    if (err != cudaSuccess) return err;
+    return launch_pdl(k, p.sms, p.nphi / 16, fr->ring_rows_smem, st, (const float4*)(adjoint ? p.wa : p.wb),
+                      (const float*)(adjoint ? p.wpre : p.wpost), y0, y1, p.nu, (const float2*)p.tw, p.err);
+}
+
 static cudaError_t launch_ring_cols(const PlanView& p, RingColsFn k, bool adjoint, cudaStream_t st)
 {
     const size_t smem = ring_cols_smem_bytes(p.nu);
@@ -2636,6 +2823,8 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
         PassRange range_("sg forward rows");
         if (sizeof(T) == 4 && p.tcm) {
             if ((err = launch_dft_r2c(p, (const float*)sigma, st)) != cudaSuccess) return err;
+        } else if (p.pairs && !sigma_direct && ring_rows_fit(p, fr, 4, wedge_row)) {
+            if ((err = launch_ring_r2c(p, fr, false, (const float*)sigma, nullptr, st)) != cudaSuccess) return err;
         } else if (p.pairs) {
             const FixedRowKernels& rk = fr->pick(p.nu, 4, p.sms);
             const int nblk = p.nu / (4 * rk.slots);
@@ -2712,6 +2901,8 @@ cudaError_t launch_forward(const PlanView& p0, const T* sigma, T* Fr, T* Fp, cud
         PassRange range_("sg forward inverse rows");
         if (sizeof(T) == 4 && p.tcm) {
             if ((err = launch_dft_c2r(p, (float*)Fr, (float*)Fp, st)) != cudaSuccess) return err;
+        } else if (p.pairs && ring_rows_fit(p, fr, 2, false)) {
+            if ((err = launch_ring_c2r(p, fr, false, (float*)Fr, (float*)Fp, st)) != cudaSuccess) return err;
         } else if (p.pairs) {
             const FixedRowKernels& rk = fr->pick(p.nu, 2, p.sms);
             const int nblk = p.nu / (2 * rk.slots);
@@ -2766,6 +2957,8 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
         PassRange range_("sg adjoint rows");
         if (sizeof(T) == 4 && p.tcm) {
             if ((err = launch_dft_r2c_adjoint(p, (const float*)gr, (const float*)gp, st)) != cudaSuccess) return err;
+        } else if (p.pairs && ring_rows_fit(p, fr, 2, false)) {
+            if ((err = launch_ring_r2c(p, fr, true, (const float*)gr, (const float*)gp, st)) != cudaSuccess) return err;
         } else if (p.pairs) {  // (A, C) pairs into wb
             const FixedRowKernels& rk = fr->pick(p.nu, 2, p.sms);
             const int nblk = p.nu / (2 * rk.slots);
@@ -2840,6 +3033,8 @@ cudaError_t launch_backward(const PlanView& p0, const T* gr, const T* gp, T* gs,
         PassRange range_("sg adjoint inverse rows");
         if (sizeof(T) == 4 && p.tcm) {
             if ((err = launch_dft_c2r_adjoint(p, (float*)gs, st)) != cudaSuccess) return err;
+        } else if (p.pairs && ring_rows_fit(p, fr, 4, wedge_done)) {
+            if ((err = launch_ring_c2r(p, fr, true, (float*)gs, nullptr, st)) != cudaSuccess) return err;
         } else if (p.pairs) {  // B from wa
             const FixedRowKernels& rk = fr->pick(p.nu, 4, p.sms);
             const int nblk = p.nu / (4 * rk.slots);
