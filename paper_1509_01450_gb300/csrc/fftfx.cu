@@ -67,7 +67,7 @@ cudaError_t launch_fx_c2r(const PlanView& p, double* y0, double* y1, cudaStream_
                       y1, p.nu, (const fxw*)p.twx, p.err, m[1], m[2]);
 }
 
-size_t fx_twiddle_bytes() { return (size_t)fx_tw_entries() * sizeof(fxw); }
+size_t fx_twiddle_bytes() { return (size_t)(FX_SMAX - FX_SMIN + 1) * fx_tw_entries() * sizeof(fxw); }
 const void* fx_twiddles()
 {
     static const std::vector<fxw> table = fx_twiddle_table();  // made once, thread-safe

@@ -11,14 +11,17 @@
 // twiddles come from tables laid out by pass (fx_tw_base), read through L1:
 // their 61 bits would cost more to form by products.
 //
-// What bounds them: instruction issue, and before that the instruction cache.
-// A complex product is some 55 instructions, so unrolled passes are long: with
+// What bounds them: the integer pipes (a complex product is twelve wide
+// multiply-adds and some fifteen additions and moves), and before that the
+// instruction cache: unrolled passes are long, and with
 // 16 points per thread, every pass unrolled and the inverse transforms apart
 // (140 KB of code in the column kernel) half of the cycles waited for
 // instructions.  Here the radix-8 passes of a kernel are one loop, and the
 // column kernels' three transforms share it (inverses as conj FFT conj).
 // Measured at 1024 x 2048, the FP64 pipe's kernels -> these, us: R2C rows 105
-// -> 32, columns 486 -> 111, C2R rows 195 -> 55; a forward call 781 -> 188.
+// -> 31, columns 486 -> 99, C2R rows 195 -> 52; a forward call 781 -> 171.
+// Products that shifted their sums into place, and whose digits' products the
+// compiler widened to 64 x 64 bits, took 32, 111, 55 and 188.
 // Error of F_phi on a smooth disk of 256 x 512 against an 80-bit evaluation:
 // 1.6e-15 -> 1.6e-16 (F_r 4.4e-16 -> 2.2e-16).
 #pragma once
@@ -39,6 +42,10 @@ struct FxShape {
 // registers); 512-thread blocks two (64 registers) where shared memory holds two
 constexpr int fx_minb(int threads, size_t smem) { return threads > 512 || 2 * smem > 220 * 1024 ? 1 : threads == 512 ? 2 : 768 / threads; }
 
+// twiddles of a pass loaded before its second barrier, of seven (1024 x 2048
+// forward call, us: none 173.5, 2: 171.5, 3: 171.6, 4: 170.7; more spill)
+constexpr int FX_AHEAD = 4;
+
 // OR / maximum over one transform's threads (whole warps) into a shared word, zero before
 __device__ __forceinline__ void fx_or_into(unsigned f, unsigned* word)
 {
@@ -55,6 +62,15 @@ __device__ __forceinline__ fx2 fx_ldg(const fx2* p)
 {
     const longlong2 v = __ldg(reinterpret_cast<const longlong2*>(p));
     return fx2{v.x, v.y};
+}
+// loaded where it stands (ahead of a barrier)
+__device__ __forceinline__ fxw fx_ldg_here(const fxw* p)
+{
+    fxw v;
+    asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.rh), "=r"(v.rl), "=r"(v.ih), "=r"(v.il)
+                 : "l"(p));
+    return v;
 }
 __device__ __forceinline__ fxw fx_ldg(const fxw* p)
 {
@@ -91,28 +107,37 @@ __device__ __forceinline__ void fx_fft(fx2 (&v)[8], fx2* sm, unsigned* nrm, int 
     const fxw* w = tw + fx_tw_base(LG, 0);
 #pragma unroll 1
     for (int p = 0; p < NP; p++) {
-        unsigned f = 0;
-#pragma unroll
-        for (int e = 0; e < 8; e++) f |= fx_fold(v[e]);
-        fx_or_into(f, nrm + p);
+        fx_or_into(fx_fold(v), nrm + p);
         if (p > 0) {
-            const int Np = Ns >> 3, k = t & (Np - 1), base = (t - k) * 8 + k;
+            // base's low digits are k < Np: the padding of r Np adds to base's
+            const int Np = Ns >> 3, k = t & (Np - 1);
+            fx2* const q = sm + sg_pad((t - k) * 8 + k);
 #pragma unroll
-            for (int r = 0; r < 8; r++) sm[sg_pad(base + r * Np)] = v[r];
+            for (int r = 0; r < 8; r++) q[sg_pad(r * Np)] = v[r];
         }
-        const int k = t & (Ns - 1);
         __syncthreads();
-        const int s = max(fx_bits(nrm[p]) - FX_T, 0);
+        int s = max(fx_bits(nrm[p]) - FX_T, 0);
 #pragma unroll
         for (int r = 0; r < 8; r++) v[r] = sm[sg_pad(t) + r * (NT + NT / 16)];
+        // the table for a shift of s, and the first twiddles ahead of the barrier
+        const fxw* q = w + (max(s, FX_SMIN) - FX_SMIN) * fx_tw_entries() + (t & (Ns - 1));
+        fxw ahead[FX_AHEAD];
+#pragma unroll
+        for (int r = 0; r < FX_AHEAD; r++) ahead[r] = fx_ldg_here(q + r * Ns);
         __syncthreads();
         E += s;
-        const long long rnd = fx_round(s), h = s > 0 ? 1ll << (s - 1) : 0;
+        if (s < FX_SMIN) {
+            const int up = FX_SMIN - s;
+#pragma unroll
+            for (int r = 0; r < 8; r++) v[r] = fx2{v[r].x << up, v[r].y << up};
+            s = FX_SMIN;
+        }
+        const long long h = 1ll << (s - 1);
         v[0] = fx2{(v[0].x + h) >> s, (v[0].y + h) >> s};
 #pragma unroll
-        for (int r = 1; r < 8; r++) {
-            v[r] = fx_cmul<DIR>(v[r], fx_ldg(w + (r - 1) * Ns + k), s, rnd);
-        }
+        for (int r = 1; r <= FX_AHEAD; r++) v[r] = fx_cmul<DIR>(v[r], ahead[r - 1]);
+#pragma unroll
+        for (int r = FX_AHEAD + 1; r < 8; r++) v[r] = fx_cmul<DIR>(v[r], fx_ldg(q + (r - 1) * Ns));
         fx_dft<8, DIR>(v);
         w += 7 * Ns;
         Ns <<= 3;
@@ -319,11 +344,11 @@ __device__ __forceinline__ fx2 fx_operand(fx2 a, const fx2* sm, int k, bool z)
     if (!SECOND) return fx2{(a.x >> 1) + (b.x >> 1), (a.y >> 1) - (b.y >> 1)};
     return fx2{(a.y >> 1) + (b.y >> 1), (b.x >> 1) - (a.x >> 1)};
 }
-// DIR < 0: a K, DIR > 0: a conj K; at 2^-60 of the factors' scale
+// DIR < 0: a K, DIR > 0: a conj K; at 2^-64 of the factors' scale
 template <int DIR>
 __device__ __forceinline__ fx2 fx_product(fx2 a, fx2 w, int dE, unsigned& top)
 {
-    const fx2 p = fx_cmul<DIR>(a, fx_digits(w.x, w.y), 0, fx_round(0));
+    const fx2 p = fx_cmul<DIR>(a, fx_digits(w.x, w.y));
     top = max(top, (unsigned)(fx_bits(fx_fold(p)) + 64 - dE));
     return p;
 }
@@ -447,13 +472,13 @@ __global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
                 v[e] = fx_conj(fx2{a.x - b.y, a.y + b.x});
                 park[t + e * NT] = fx2{0, 0};
             }
-            E2 = E = E + EK + q + FX_WBITS - FX_T;
+            E2 = E = E + EK + q + FX_PROD - FX_T;
         } else {
 #pragma unroll
             for (int e = 0; e < 8; e++) v[e] = fx_conj(fx_align<NT, false>(v[e], K, t, e, q1 - FX_T));
-            E2 = E + EK2 + q2 + FX_WBITS - FX_T;
+            E2 = E + EK2 + q2 + FX_PROD - FX_T;
             shift2 = q2 - FX_T;
-            E = E + EK1 + q1 + FX_WBITS - FX_T;
+            E = E + EK1 + q1 + FX_PROD - FX_T;
         }
     }
 }
@@ -506,7 +531,7 @@ __global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
                 park[k] = fx_product<+1>(fx_operand<LG, false>(v[e], sm, k, K.z), w, d, top);
             }
             fx_max_into(top, &nrm[slot][11]);
-            Ep0 = E + (int)fx_ldg(K.k1 + nu + 1).x + FX_WBITS - FX_T;
+            Ep0 = E + (int)fx_ldg(K.k1 + nu + 1).x + FX_PROD - FX_T;
             __syncthreads();  // every mirror read is done
             fx_load_column<NT>(v, (K.z ? A : C) + (size_t)m * nu + t, &nrm[slot][10], E);
         } else {
@@ -520,7 +545,7 @@ __global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
             __syncthreads();  // every mirror read is done; the largest products are known
             // both products at the larger one's exponent, one bit of room for their sum
             const int q1 = (int)nrm[slot][11] - 64, q2 = (int)nrm[slot][12] - 64;
-            const int Ep1 = E + (int)fx_ldg(K.k2 + nu + 1).x + FX_WBITS - FX_T;
+            const int Ep1 = E + (int)fx_ldg(K.k2 + nu + 1).x + FX_PROD - FX_T;
             E = max(Ep0 + q1, Ep1 + q2) + 1;
             const int s1 = E - Ep0 - FX_T, s2 = E - Ep1 - FX_T;
 #pragma unroll

@@ -17,13 +17,15 @@
 // twiddle products shift by what it grew (s <= 4).  The largest modulus never
 // shrinks through an orthogonal pass, so no shift to the left is needed.
 //
-// Products.  A factor w of modulus <= 1 is held as 2^60 w; both operands are
-// split in signed 32-bit digits a = ah 2^32 + al, and
-//   a w 2^-60 = (ah wh) 2^4 + (ah wl + al wh) 2^-28
-// without al wl (0.3 units rms).  The digit products accumulate in 64 bits
-// over a complex product's two terms, so that its parts take six multiply-adds
-// and one shift each; Karatsuba's three real products would save three of the
-// twelve multiply-adds for seven more additions, digits and one bit of headroom.
+// Products.  Both operands are split in signed 32-bit digits a = ah 2^32 + al,
+// and with the factor w held as W = 2^(64 - s) w
+//   a w 2^-s = a W 2^-64 = ah Wh + (ah Wl + al Wh) 2^-32
+// without al Wl (a quarter of a unit at most).  The digit products accumulate
+// in 64 bits over a complex product's two terms, so that its parts take six
+// multiply-adds and one addition of a high word each, no shifts: the twiddles
+// are tabled for s = 2, 3, 4, and a block that grew by less is moved up first
+// (s = 2).  Karatsuba's three real products would save three of the twelve
+// multiply-adds for seven more additions, digits and one bit of headroom.
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -39,38 +41,54 @@ struct __align__(16) fx2 {
 namespace sg {
 
 constexpr int FX_T = 59;      // bits of the largest component before a pass
-constexpr int FX_WBITS = 60;  // scale of the twiddles
+constexpr int FX_PROD = 64;              // a product's scale below its factors'
+constexpr int FX_SMIN = 2, FX_SMAX = 4;  // a product's shifts s
 
 FXHD int fx_h(long long a) { return (int)(a >> 32) + (int)((unsigned)a >> 31); }
 FXHD int fx_l(long long a) { return (int)(unsigned)a; }
-FXHD long long fx_wide(int a, int b, long long c) { return (long long)a * b + c; }
+// a b + c, as one instruction: left to the compiler, a negated digit is
+// widened before its sign is changed, and its product becomes one of 64 x 64 bits
+FXHD long long fx_wide(int a, int b, long long c)
+{
+#ifdef __CUDA_ARCH__
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+#else
+    return (long long)((unsigned long long)((long long)a * b) + (unsigned long long)c);
+#endif
+}
 
-// (hi 2^4 + mid 2^-28) 2^-s, 0 <= s <= 4; the caller's mid starts at fx_round(s)
-FXHD long long fx_round(int s) { return 1ll << (27 + s); }
-FXHD long long fx_join(long long hi, long long mid, int s) { return (hi << (4 - s)) + (mid >> (28 + s)); }
+// hi + mid 2^-32, rounded: the sums start at FX_HI and FX_MID, which hold the
+// rounding and 2^63 more in mid, so that its high word is added unsigned
+constexpr long long FX_MID = (long long)(0x8000000080000000ull), FX_HI = -(1ll << 31);
+FXHD long long fx_join(long long hi, long long mid) { return hi + (long long)((unsigned long long)mid >> 32); }
 
-// a factor's digits: 2^60 w = (rh + i ih) 2^32 + (rl + i il), no digit -2^31
+// a factor's digits: W = (rh + i ih) 2^32 + (rl + i il), no digit -2^31
 struct __align__(16) fxw {
     int rh, rl, ih, il;
 };
 FXHD fxw fx_digits(long long wr, long long wi) { return fxw{fx_h(wr), fx_l(wr), fx_h(wi), fx_l(wi)}; }
-// a w 2^-(60 + s) (DIR < 0) or a conj(w) 2^-(60 + s) (DIR > 0); |a| <= 2^62.5, |w| <= 2^60
+// a W 2^-64 (DIR < 0) or a conj(W) 2^-64 (DIR > 0).  The middle sums stay
+// below 2^63: |ah| sqrt 2 2^31 + sqrt 2 2^31 |Wh| with |a| <= 2^(59.5 + s),
+// |W| <= 2^(64 - s) for a twiddle, |a| <= 2^62.5, |W| <= 2^61.5 for a spectrum
 template <int DIR>
-FXHD fx2 fx_cmul(fx2 a, fxw w, int s, long long rnd)
+FXHD fx2 fx_cmul(fx2 a, fxw w)
 {
     const int xh = fx_h(a.x), xl = fx_l(a.x), yh = fx_h(a.y), yl = fx_l(a.y);
     const int uh = DIR < 0 ? -w.ih : w.ih, ul = DIR < 0 ? -w.il : w.il;  // times y, into the real part
     const int vh = DIR < 0 ? w.ih : -w.ih, vl = DIR < 0 ? w.il : -w.il;  // times x, into the imaginary part
-    const long long rm = fx_wide(xl, w.rh, fx_wide(xh, w.rl, fx_wide(yl, uh, fx_wide(yh, ul, rnd))));
-    const long long im = fx_wide(yl, w.rh, fx_wide(yh, w.rl, fx_wide(xl, vh, fx_wide(xh, vl, rnd))));
-    return fx2{fx_join(fx_wide(xh, w.rh, fx_wide(yh, uh, 0)), rm, s),
-               fx_join(fx_wide(yh, w.rh, fx_wide(xh, vh, 0)), im, s)};
+    const long long rm = fx_wide(xl, w.rh, fx_wide(xh, w.rl, fx_wide(yl, uh, fx_wide(yh, ul, FX_MID))));
+    const long long im = fx_wide(yl, w.rh, fx_wide(yh, w.rl, fx_wide(xl, vh, fx_wide(xh, vl, FX_MID))));
+    return fx2{fx_join(fx_wide(xh, w.rh, fx_wide(yh, uh, FX_HI)), rm),
+               fx_join(fx_wide(yh, w.rh, fx_wide(xh, vh, FX_HI)), im)};
 }
-// a times the real constant r (2^60 r given)
-FXHD long long fx_rmul(long long a, long long r)
+// a / sqrt 2, as a - a (1 - 1 / sqrt 2): that factor fits 2^64 times itself
+FXHD long long fx_rmul(long long a)
 {
+    constexpr long long r = 0x4AFB0CCC06219B7Cll;  // round(2^64 (1 - 1 / sqrt 2))
     const int ah = fx_h(a), al = fx_l(a), rh = fx_h(r), rl = fx_l(r);
-    return fx_join(fx_wide(ah, rh, 0), fx_wide(al, rh, fx_wide(ah, rl, fx_round(0))), 0);
+    return a - fx_join(fx_wide(ah, rh, FX_HI), fx_wide(al, rh, fx_wide(ah, rl, FX_MID)));
 }
 
 FXHD fx2 fx_add(fx2 a, fx2 b) { return fx2{a.x + b.x, a.y + b.y}; }
@@ -92,9 +110,8 @@ FXHD void fx_dft4(fx2& a0, fx2& a1, fx2& a2, fx2& a3)
 template <int DIR, int K>
 FXHD fx2 fx_w8(fx2 a)
 {
-    const long long r = 0x0B504F333F9DE648ll;  // round(2^60 / sqrt 2)
-    if (K == 1) return fx2{fx_rmul(a.x - DIR * a.y, r), fx_rmul(a.y + DIR * a.x, r)};
-    return fx2{fx_rmul(-a.x - DIR * a.y, r), fx_rmul(-a.y + DIR * a.x, r)};
+    if (K == 1) return fx2{fx_rmul(a.x - DIR * a.y), fx_rmul(a.y + DIR * a.x)};
+    return fx2{fx_rmul(-a.x - DIR * a.y), fx_rmul(-a.y + DIR * a.x)};
 }
 template <int R, int DIR>
 FXHD void fx_dft(fx2* a)
@@ -140,15 +157,33 @@ FXHD int fx_clz64(unsigned long long v)
     return v ? __builtin_clzll(v) : 64;
 #endif
 }
+// the same bound for eight values, from the extremes of their high words
+FXHD unsigned fx_fold(const fx2 (&v)[8])
+{
+    int hi = (int)(v[0].x >> 32), lo = hi;
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        const int a = (int)(v[e].x >> 32), b = (int)(v[e].y >> 32);
+#ifdef __CUDA_ARCH__
+        hi = __vimax3_s32(hi, a, b);
+        lo = __vimin3_s32(lo, a, b);
+#else
+        hi = hi > a ? hi : a;
+        hi = hi > b ? hi : b;
+        lo = lo < a ? lo : a;
+        lo = lo < b ? lo : b;
+#endif
+    }
+    return (unsigned)(hi > ~lo ? hi : ~lo);
+}
 // bits of the block's largest component from the OR of fx_fold
 FXHD int fx_bits(unsigned folded) { return 64 - fx_clz32(folded); }
 
-// x 2^-d, rounded (d >= 64 gives 0), or x 2^-d for d < 0
+// x 2^-d, rounded, or x 2^-d for d < 0; |x| <= 2^62, so that d >= 63 gives 0
 FXHD long long fx_shift(long long x, int d)
 {
-    if (d <= 0) return x << (d > -63 ? -d : 63);
-    if (d > 62) return 0;
-    return (x + (1ll << (d - 1))) >> d;
+    const int l = d > 0 ? 0 : d > -63 ? -d : 63, r = d < 0 ? 0 : d < 63 ? d : 63;
+    return ((x << l) + (long long)((1ull << r) >> 1)) >> r;
 }
 
 FXHD unsigned long long fx_dbits(double d)
@@ -217,8 +252,8 @@ FXHD double fx_to_double_any(long long x, int E)
 // ---------------------------------------------------------------------------
 // Kernel spectra in fixed point: per mode m a row of N_u + 2 entries, kappa =
 // 0 .. N_u and the row's exponent.  Entry kappa holds (x, y) with K = (x + i
-// y) 2^(e_row - dE): |x|, |y| <= 2^59, dE in 0..63 in the low three bits of x
-// and y (57 bits below the entry's own modulus are left, rounded).
+// y) 2^(e_row - dE): |x|, |y| <= 2^61, dE in 0..63 in the low three bits of x
+// and y (59 bits below the entry's own modulus are left, rounded).
 // ---------------------------------------------------------------------------
 FXHD long long fx_spec_round(long long x)
 {
@@ -232,17 +267,18 @@ FXHD fx2 fx_spec_entry(double kx, double ky, int Frow)
     int dE = Frow - f;
     dE = dE > 63 ? 63 : dE;
     const int F = Frow - dE;  // >= f
-    const long long x = fx_from_double(kx, F), y = fx_from_double(ky, F);
+    const long long x = fx_from_double(kx, F) * 4, y = fx_from_double(ky, F) * 4;
     return fx2{fx_spec_round(x) | (dE & 7), fx_spec_round(y) | (dE >> 3)};
 }
 FXHD int fx_spec_drop(fx2 w) { return ((int)w.x & 7) | ((int)w.y & 7) << 3; }  // dE
 FXHD fx2 fx_spec_mant(fx2 w) { return fx2{w.x & ~7ll, w.y & ~7ll}; }
-FXHD int fx_spec_exp(int Frow) { return fx_exp_of_field(Frow); }  // e_row: K = x 2^(e_row - dE)
+FXHD int fx_spec_exp(int Frow) { return fx_exp_of_field(Frow) - 2; }  // e_row: K = x 2^(e_row - dE)
 
 // twiddle tables: for a transform of 2^LG points the radix-8 passes after the
 // first (radix 2, 4 or 8) take w^r, w = e^{-2 pi i k / (8 Ns)}, k < Ns the
 // place in the Ns points done before, at fx_tw_base(LG, pass) + (r - 1) Ns +
-// k, so that a warp's loads of one power are contiguous
+// k, so that a warp's loads of one power are contiguous; one such table for
+// each shift s, fx_tw_entries() apart
 constexpr int FX_MIN_LG = 8, FX_MAX_LG = 12;
 FXHD constexpr int fx_first_lg(int LG) { return LG % 3 ? LG % 3 : 3; }
 FXHD constexpr int fx_passes(int LG) { return (LG - 1) / 3; }  // radix-8 passes after the first
@@ -258,7 +294,7 @@ FXHD constexpr int fx_tw_base(int LG, int pass)
 }
 FXHD constexpr int fx_tw_entries() { return fx_tw_base(FX_MAX_LG, 99); }
 
-// 2^60 (cos, sin) of 2 pi j / 4096, j = 0 .. 512, rounded: Taylor series in
+// 2^62 (cos, sin) of 2 pi j / 4096, j = 0 .. 512, rounded: Taylor series in
 // double-double (two-term sums and FMA products), good to about 2^-100.
 // Twiddles rounded at 53 bits would leak 2^-54 of a strong mode into all
 // others, several times what the transforms' own rounding leaves.
@@ -286,7 +322,11 @@ inline std::vector<long long> fx_octant()
             const double q = h / n;
             return norm(q, (fma(-q, n, h) + l) / n);
         }
-        long long fixed() const { return (long long)(h * 0x1p60) + llrint(l * 0x1p60); }  // h 2^60 is whole
+        long long fixed() const
+        {
+            const double a = h * 0x1p62, whole = floor(a);
+            return (long long)whole + llrint((a - whole) + l * 0x1p62);
+        }
     };
     std::vector<long long> t(2 * 513);
     const dd step = dd{0x1.921fb54442d18p-10, 0x1.1a62633145c07p-64};  // pi / 2048
@@ -304,11 +344,11 @@ inline std::vector<long long> fx_octant()
     }
     return t;
 }
-// the twiddle tables (fx_tw_entries() factors)
+// the twiddle tables ((FX_SMAX - FX_SMIN + 1) fx_tw_entries() factors)
 inline std::vector<fxw> fx_twiddle_table()
 {
     const std::vector<long long> q = fx_octant();
-    std::vector<fxw> out(fx_tw_entries());
+    std::vector<fxw> out((FX_SMAX - FX_SMIN + 1) * fx_tw_entries());
     for (int lg = FX_MIN_LG; lg <= FX_MAX_LG; lg++)
         for (int p = 0; p < fx_passes(lg); p++) {
             const int ns = 1 << (fx_first_lg(lg) + 3 * p);
@@ -317,10 +357,13 @@ inline std::vector<fxw> fx_twiddle_table()
                     const int j = r * k * (4096 / (8 * ns)) & 4095, o = j >> 9, i = j & 511;  // octant, place in it
                     const long long *e = &q[2 * ((o & 1) ? 512 - i : i)], c = (o + 1) & 2 ? e[1] : e[0],
                                     s = (o + 1) & 2 ? e[0] : e[1];
-                    long long x = o >= 2 && o <= 5 ? -c : c, y = o >= 4 ? s : -s;  // cos, -sin of 2 pi j / 4096
-                    x += fx_l(x) == INT32_MIN;  // no low digit of -2^31
-                    y += fx_l(y) == INT32_MIN;
-                    out[fx_tw_base(lg, p) + (r - 1) * ns + k] = fx_digits(x, y);
+                    const long long wr = o >= 2 && o <= 5 ? -c : c, wi = o >= 4 ? s : -s;  // cos, -sin of 2 pi j / 4096
+                    for (int t = FX_SMIN; t <= FX_SMAX; t++) {
+                        long long x = fx_shift(wr, t - 2), y = fx_shift(wi, t - 2);
+                        x += fx_l(x) == INT32_MIN;  // no low digit of -2^31
+                        y += fx_l(y) == INT32_MIN;
+                        out[(t - FX_SMIN) * fx_tw_entries() + fx_tw_base(lg, p) + (r - 1) * ns + k] = fx_digits(x, y);
+                    }
                 }
         }
     return out;
