@@ -180,8 +180,8 @@ sg_status sg_plan_create(sg_plan** out, int nu, int nphi, double u_min, double d
         (st = dev_alloc(p, (void**)&p->cells, (size_t)6 * (2 * nu + 1) * nphi * sizeof(double))) ||
         (st = dev_alloc(p, (void**)&p->keff, (size_t)2 * (2 * nu - 1) * nphi * sizeof(double))) ||
         // the fixed-point passes' tables, where either direction has such transforms
-        (dtype != SG_F32 && (nphi >= 256 || nu >= 128) && (st = dev_alloc(p, &p->twx, fx_twiddle_bytes()))) ||
-        (dtype != SG_F32 && nu >= 128 &&
+        (dtype != SG_F32 && (nphi >= 64 || nu >= 32) && (st = dev_alloc(p, &p->twx, fx_twiddle_bytes()))) ||
+        (dtype != SG_F32 && nu >= 32 &&
          ((st = dev_alloc(p, &p->kfr, nk * 16)) || (st = dev_alloc(p, &p->kfp, nk * 16)))) ||
         (dtype == SG_F32X2 && ((st = dev_alloc(p, &p->xf, (size_t)3 * nu * nphi * sizeof(dfloat))) ||
                                (st = dev_alloc(p, &p->xw, (size_t)2 * nphi * sizeof(dfloat)))))) {

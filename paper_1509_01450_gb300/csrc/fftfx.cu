@@ -7,8 +7,8 @@ namespace sg {
 
 static const FxKernels* fx_kernels(int n)
 {
-    static const FxKernels table[5] = {fx_kernels_lg8(), fx_kernels_lg9(), fx_kernels_lg10(), fx_kernels_lg11(),
-                                       fx_kernels_lg12()};
+    static const FxKernels table[] = {fx_kernels_lg6(), fx_kernels_lg7(),  fx_kernels_lg8(), fx_kernels_lg9(),
+                                      fx_kernels_lg10(), fx_kernels_lg11(), fx_kernels_lg12()};
     const int lg = sg_ilog2(n);
     return lg >= FX_MIN_LG && lg <= FX_MAX_LG ? &table[lg - FX_MIN_LG] : nullptr;
 }

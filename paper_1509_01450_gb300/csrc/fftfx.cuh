@@ -34,7 +34,7 @@ template <int LG>
 struct FxShape {
     static constexpr int N = 1 << LG, NT = N / 8;
     static constexpr int SL = NT >= 128 ? 1 : 128 / NT;  // transforms per block: R2C rows, columns
-    static constexpr int RB = NT >= 64 ? 2 : 4;          // rows per block where 32-byte sectors need two
+    static constexpr int RB = NT >= 64 ? 2 : 128 / NT;  // rows per block where 32-byte sectors need two (one of the tensor maps' two)
     static constexpr size_t EX = (size_t)(N + N / 16 + 1) * sizeof(fx2);  // one exchange area
     static constexpr size_t PARK = (size_t)N * sizeof(fx2);               // one parked spectrum
 };
@@ -46,16 +46,28 @@ constexpr int fx_minb(int threads, size_t smem) { return threads > 512 || 2 * sm
 // forward call, us: none 173.5, 2: 171.5, 3: 171.6, 4: 170.7; more spill)
 constexpr int FX_AHEAD = 4;
 
-// OR / maximum over one transform's threads (whole warps) into a shared word, zero before
+// OR / maximum over one transform's NT threads (whole warps, or 8 or 16 lanes) into a shared word, zero before
+template <int NT>
 __device__ __forceinline__ void fx_or_into(unsigned f, unsigned* word)
 {
-    f = __reduce_or_sync(0xffffffffu, f);
-    if ((threadIdx.x & 31) == 0) atomicOr(word, f);
+    if constexpr (NT >= 32) {
+        f = __reduce_or_sync(0xffffffffu, f);
+    } else {
+#pragma unroll
+        for (int o = NT / 2; o > 0; o >>= 1) f |= __shfl_xor_sync(0xffffffffu, f, o);
+    }
+    if ((threadIdx.x & (NT < 32 ? NT - 1 : 31)) == 0) atomicOr(word, f);
 }
+template <int NT>
 __device__ __forceinline__ void fx_max_into(unsigned f, unsigned* word)
 {
-    f = __reduce_max_sync(0xffffffffu, f);
-    if ((threadIdx.x & 31) == 0) atomicMax(word, f);
+    if constexpr (NT >= 32) {
+        f = __reduce_max_sync(0xffffffffu, f);
+    } else {
+#pragma unroll
+        for (int o = NT / 2; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
+    }
+    if ((threadIdx.x & (NT < 32 ? NT - 1 : 31)) == 0) atomicMax(word, f);
 }
 
 __device__ __forceinline__ fx2 fx_ldg(const fx2* p)
@@ -107,7 +119,7 @@ __device__ __forceinline__ void fx_fft(fx2 (&v)[8], fx2* sm, unsigned* nrm, int 
     const fxw* w = tw + fx_tw_base(LG, 0);
 #pragma unroll 1
     for (int p = 0; p < NP; p++) {
-        fx_or_into(fx_fold(v), nrm + p);
+        fx_or_into<NT>(fx_fold(v), nrm + p);
         if (p > 0) {
             // base's low digits are k < Np: the padding of r Np adds to base's
             const int Np = Ns >> 3, k = t & (Np - 1);
@@ -118,7 +130,7 @@ __device__ __forceinline__ void fx_fft(fx2 (&v)[8], fx2* sm, unsigned* nrm, int 
         __syncthreads();
         int s = max(fx_bits(nrm[p]) - FX_T, 0);
 #pragma unroll
-        for (int r = 0; r < 8; r++) v[r] = sm[sg_pad(t) + r * (NT + NT / 16)];
+        for (int r = 0; r < 8; r++) v[r] = sm[sg_pad(t) + sg_pad(r * NT)];
         // the table for a shift of s, and the first twiddles ahead of the barrier
         const fxw* q = w + (max(s, FX_SMIN) - FX_SMIN) * fx_tw_entries() + (t & (Ns - 1));
         fxw ahead[FX_AHEAD];
@@ -221,7 +233,7 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
     for (int e = 0; e < 8; e++) h = max(h, max(fx_abshi(z[e].x), fx_abshi(z[e].y)));
     if (t == 0) level[slot] = z[0];
     __syncthreads();
-    fx_max_into(h, &nrm[slot][3]);
+    fx_max_into<NT>(h, &nrm[slot][3]);
     __syncthreads();
     h = nrm[slot][3];
     const int F = fx_field(h);
@@ -237,7 +249,7 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
         v[e] = fx2{fx_from_double(z[e].x, F) - c.x, fx_from_double(z[e].y, F) - c.y};
         g |= fx_fold(v[e]);
     }
-    fx_or_into(g, &nrm[slot][4]);
+    fx_or_into<NT>(g, &nrm[slot][4]);
     __syncthreads();
     const int up = FX_T - fx_bits(nrm[slot][4]);
 #pragma unroll
@@ -380,7 +392,7 @@ __device__ __forceinline__ void fx_load_column(fx2 (&v)[8], const double2* __res
     for (int e = 0; e < 4; e++) a[e] = sg_ld_dep(in + e * NT);
 #pragma unroll
     for (int e = 0; e < 4; e++) h = max(h, max(fx_abshi(a[e].x), fx_abshi(a[e].y)));
-    fx_max_into(h, top);
+    fx_max_into<NT>(h, top);
     __syncthreads();
     h = *top;
     const int F = fx_field(h);
@@ -418,7 +430,7 @@ __global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
     const int slot = threadIdx.x / NT, t = threadIdx.x % NT;
     fx2* const sm = reinterpret_cast<fx2*>(smraw) + (size_t)slot * (L + L / 16 + 1);
     fx2* const park = reinterpret_cast<fx2*>(smraw + SL * FxShape<LG>::EX) + (size_t)slot * L;
-    if (t < 12) nrm[slot][t] = 0;
+    for (int j = t; j < 12; j += NT) nrm[slot][j] = 0;
     const int m0 = blockIdx.x * SL + slot;
     const bool live = m0 < half;
     const int m = live ? m0 : half - 1;
@@ -458,8 +470,8 @@ __global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
             const fx2 w1 = fx_spec_at<NT, false>(K, t, e, d1);
             v[e] = fx_product<-1>(fx_operand<LG, false>(v[e], sm, k, K.z), w1, d1, top1);
         }
-        fx_max_into(top1, &nrm[slot][10]);
-        fx_max_into(top2, &nrm[slot][11]);
+        fx_max_into<NT>(top1, &nrm[slot][10]);
+        fx_max_into<NT>(top2, &nrm[slot][11]);
         __syncthreads();
         const int q1 = (int)nrm[slot][10] - 64, q2 = (int)nrm[slot][11] - 64;
         const int EK1 = (int)fx_ldg(K.k1 + nu + 1).x, EK2 = (int)fx_ldg(K.k2 + nu + 1).x;
@@ -497,7 +509,7 @@ __global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
     const int slot = threadIdx.x / NT, t = threadIdx.x % NT;
     fx2* const sm = reinterpret_cast<fx2*>(smraw) + (size_t)slot * (L + L / 16 + 1);
     fx2* const park = reinterpret_cast<fx2*>(smraw + SL * FxShape<LG>::EX) + (size_t)slot * L;
-    if (t < 13) nrm[slot][t] = 0;
+    for (int j = t; j < 13; j += NT) nrm[slot][j] = 0;
     const int m0 = blockIdx.x * SL + slot;
     const bool live = m0 < half;
     const int m = live ? m0 : half - 1;
@@ -530,7 +542,7 @@ __global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
                 const fx2 w = fx_spec_at<NT, false>(K, t, e, d);
                 park[k] = fx_product<+1>(fx_operand<LG, false>(v[e], sm, k, K.z), w, d, top);
             }
-            fx_max_into(top, &nrm[slot][11]);
+            fx_max_into<NT>(top, &nrm[slot][11]);
             Ep0 = E + (int)fx_ldg(K.k1 + nu + 1).x + FX_PROD - FX_T;
             __syncthreads();  // every mirror read is done
             fx_load_column<NT>(v, (K.z ? A : C) + (size_t)m * nu + t, &nrm[slot][10], E);
@@ -541,7 +553,7 @@ __global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
                 const fx2 w = fx_spec_at<NT, true>(K, t, e, d);
                 v[e] = fx_product<+1>(fx_operand<LG, true>(v[e], sm, t + e * NT, K.z), w, d, top);
             }
-            fx_max_into(top, &nrm[slot][12]);
+            fx_max_into<NT>(top, &nrm[slot][12]);
             __syncthreads();  // every mirror read is done; the largest products are known
             // both products at the larger one's exponent, one bit of room for their sum
             const int q1 = (int)nrm[slot][11] - 64, q2 = (int)nrm[slot][12] - 64;
@@ -624,7 +636,7 @@ __global__ void __launch_bounds__(FxC2R<LG, BWD>::THREADS, FxC2R<LG, BWD>::MINB)
             if (e == 0 && t == 0) a[0].x = b[0].x = 0.0;
             h = max(h, max(max(fx_abshi(a[e].x), fx_abshi(a[e].y)), max(fx_abshi(b[e].x), fx_abshi(b[e].y))));
         }
-        fx_max_into(h, &nrm[slot][3]);
+        fx_max_into<NT>(h, &nrm[slot][3]);
         __syncthreads();
         h = nrm[slot][3];
         const int F = fx_field(h) + 1;  // one bit of room: Z adds two of them
@@ -709,6 +721,8 @@ FxKernels make_fx_kernels()
                      FxShape<LG>::SL,
                      FxShape<LG>::RB};
 }
+FxKernels fx_kernels_lg6();
+FxKernels fx_kernels_lg7();
 FxKernels fx_kernels_lg8();
 FxKernels fx_kernels_lg9();
 FxKernels fx_kernels_lg10();

@@ -218,8 +218,8 @@ cudaError_t launch_dft_r2c_adjoint(const PlanView& p, const float* gr, const flo
 cudaError_t launch_dft_c2r_adjoint(const PlanView& p, float* gs, cudaStream_t st);
 cudaError_t launch_dft_tc_batch(const TcArgs* d_args, int n, int dir, int max_nu, cudaStream_t st);
 // fftfx.cu: the passes in 64-bit block fixed point (sg_fx.cuh), over FP64
-// fields and FP64 half spectra.  *_ok: the plan's rows (N_phi of 256 .. 4096,
-// their tensor maps made) or columns (2 N_u of 256 .. 4096) run on them;
+// fields and FP64 half spectra.  *_ok: the plan's rows (N_phi of 64 .. 4096,
+// their tensor maps made) or columns (2 N_u of 64 .. 4096) run on them;
 // launch_fx_r2c's x1 and launch_fx_c2r's y1 are null for the forward R2C pass
 // and the adjoint C2R pass.
 bool fx_rows_ok(const PlanView& p);
