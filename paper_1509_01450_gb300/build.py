@@ -28,7 +28,7 @@ LIB_CHECKED = os.path.join(HERE, "libsgdisk_checked.so")
 # fftconv_lg<LG>.cu and fftfx_lg<LG>.cu compile the fixed-length FP32 and the
 # fixed-point pass kernels, one transform length each, in parallel with the rest
 SOURCES = ["api.cu", "batch.cu", "dft_tc.cu", "kbuild.cu", "fftconv.cu", "fftconv_df.cu", "noalloc.cu", "wedge.cu", "fftfx.cu"]
-SOURCES += [f"fftconv_lg{lg}.cu" for lg in range(8, 14)] + [f"fftfx_lg{lg}.cu" for lg in range(6, 13)]
+SOURCES += [f"fftconv_lg{lg}.cu" for lg in range(6, 14)] + [f"fftfx_lg{lg}.cu" for lg in range(6, 13)]
 HEADERS = ["sg_common.cuh", "sg_df.cuh", "sg_internal.cuh", "sg_tc.cuh", "sg_launch.cuh", "sg_fx.cuh", "fftfx.cuh", "fftconv.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -2515,14 +2515,17 @@ template <int LG>
 FixedPassKernels make_fixed_pass_kernels()
 {
     constexpr int NB = (1 << LG) / 16 > 256 ? 512 : 256;
-    FixedPassKernels k{make_fixed_row_kernels<LG, false>(),
-                       make_fixed_row_kernels<LG, (LG < 12)>(),  // one transform fills a block from 4096 points on
-                       k_fwd_cols<float, 16, NB, LG>,
-                       k_fwd_cols<float, 16, NB, LG, true>,
-                       k_fwd_cols<float, 16, NB, LG, true, true>,
-                       k_bwd_cols<float, 16, NB, LG>,
-                       k_bwd_cols<float, 16, NB, LG, true>,
-                       k_bwd_cols<float, 16, NB, LG, true, true>};
+    FixedPassKernels k{};
+    if constexpr (LG >= 8) {  // (rows of 64 and 128 points stay on the run-time instances)
+        k.rows = make_fixed_row_kernels<LG, false>();
+        k.small = make_fixed_row_kernels<LG, (LG < 12)>();  // one transform fills a block from 4096 points on
+    }
+    k.fwd_cols = k_fwd_cols<float, 16, NB, LG>;
+    k.fwd_cols_edge = k_fwd_cols<float, 16, NB, LG, true>;
+    k.fwd_cols_edge_wedge = k_fwd_cols<float, 16, NB, LG, true, true>;
+    k.bwd_cols = k_bwd_cols<float, 16, NB, LG>;
+    k.bwd_cols_edge = k_bwd_cols<float, 16, NB, LG, true>;
+    k.bwd_cols_edge_wedge = k_bwd_cols<float, 16, NB, LG, true, true>;
     if constexpr (LG > 12) {
         k.ring_cols[0] = k_ring_cols<LG, false>;
         k.ring_cols[1] = k_ring_cols<LG, true>;
@@ -2536,6 +2539,8 @@ FixedPassKernels make_fixed_pass_kernels()
 }
 
 // defined in fftconv_lg<LG>.cu
+FixedPassKernels fixed_pass_kernels_lg6();
+FixedPassKernels fixed_pass_kernels_lg7();
 FixedPassKernels fixed_pass_kernels_lg8();
 FixedPassKernels fixed_pass_kernels_lg9();
 FixedPassKernels fixed_pass_kernels_lg10();
@@ -2547,10 +2552,11 @@ FixedPassKernels fixed_pass_kernels_lg13();
 // the instances for transforms of 2^lg points, or null
 static const FixedPassKernels* fixed_pass_kernels(int lg)
 {
-    static const FixedPassKernels table[6] = {fixed_pass_kernels_lg8(),  fixed_pass_kernels_lg9(),
+    static const FixedPassKernels table[8] = {fixed_pass_kernels_lg6(),  fixed_pass_kernels_lg7(),
+                                              fixed_pass_kernels_lg8(),  fixed_pass_kernels_lg9(),
                                               fixed_pass_kernels_lg10(), fixed_pass_kernels_lg11(),
                                               fixed_pass_kernels_lg12(), fixed_pass_kernels_lg13()};
-    return lg >= 8 && lg <= 13 ? &table[lg - 8] : nullptr;
+    return lg >= 6 && lg <= 13 ? &table[lg - 6] : nullptr;
 }
 
 // ===========================================================================
@@ -2728,9 +2734,13 @@ static cudaError_t launch_edges(const PlanView& p, bool adjoint, cudaStream_t st
 }
 
 // The fixed-length instances of both transform lengths, when every pass of
-// the plan can run on them: FP32, N_phi and 2 N_u of 256 .. 8192 points, the
-// pair layout's tensor maps made, N_u a multiple of the row blocks.  The
-// passes then keep the column spectra in the pair layout.  Tensor-core rows
+// the plan can run on them: FP32, N_phi of 256 .. 8192 and 2 N_u of 64 .. 8192
+// points, the pair layout's tensor maps made, N_u a multiple of the small row
+// blocks (and then of the others where pick takes those: N_u is a power of
+// two).  The passes then keep the column spectra in the pair layout.  Columns
+// of 64 and 128 points came in for the rows' sake: the three passes of 64 x
+// 1024, launched apart, 27.6 -> 21.2 us (adjoint 30.4 -> 22.3), 32 x 8192
+// chained 36.2 -> 29.0.  Tensor-core rows
 // (short_dft) read and write that layout at any of their lengths, so with them
 // only the columns have to qualify (fr null where the rows have no instances):
 // a 4096 x 32 forward call, with the row passes chained by programmatic
@@ -2742,7 +2752,8 @@ static bool fixed_path(const PlanView& p, const FixedPassKernels*& fr, const Fix
     if (sizeof(T) != 4) return false;
     const FixedPassKernels* a = fixed_pass_kernels(sg_ilog2(p.nphi));
     const FixedPassKernels* b = fixed_pass_kernels(sg_ilog2(2 * p.nu));
-    if (!b || (!p.tcm && (!p.imaps || !a || p.nu % (4 * a->rows.slots) != 0))) return false;
+    if (a && !a->rows.slots) a = nullptr;  // columns only
+    if (!b || (!p.tcm && (!p.imaps || !a || p.nu % (4 * a->small.slots) != 0))) return false;
     fr = a;
     fc = b;
     return true;
