@@ -63,7 +63,7 @@ typedef enum {
    are stored as unevaluated sums of two FP32 numbers (about 48 significant
    bits), and the passes carry at least that: double-float arithmetic from
    error-free transformations on the FP32 pipes or, where N_phi and 2 N_u are
-   both in 2^8 .. 2^12 and neither radial_edges nor wedge is set, 64-bit block
+   both in 2^6 .. 2^12 and neither radial_edges nor wedge is set, 64-bit block
    fixed point on the integer pipes (as the SG_F64 passes of those lengths).
    Sizes as for SG_F64. */
 typedef enum { SG_F32 = 0, SG_F64 = 1, SG_F32X2 = 2 } sg_dtype;
