@@ -479,17 +479,21 @@ static sg_status make_list(const sg_batch_item* items, int n, const BatchTuning&
             b.tc_max_nu = std::max(b.tc_max_nu, p->nu);
         }
     }
-    // each pass's items, the disks' in order of decreasing work (largest
-    // first, so that the small ones fill the last wave) unless natural
-    std::vector<int> order(n);
-    for (int i = 0; i < n; i++) order[i] = i;
-    if (!tu.natural)
-        std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
-            return (long)D[a].nu * D[a].nphi > (long)D[c].nu * D[c].nphi;
-        });
+    // each pass's items, disk by disk, the largest disks first, or as given
+    // (natural).  Column items go by length before that, the longest first: the
+    // five lengths' code is more than the instruction cache holds, and so the
+    // blocks run one of them at a time (256 disks: 787 -> 772 us, the row passes
+    // unchanged by it).
     std::vector<int2> q;
     const std::vector<int>* counts[3] = {&n_rows, &n_cols, &n_inv};
     for (int k = 0; k < 3; k++) {
+        std::vector<int> order(n);
+        for (int i = 0; i < n; i++) order[i] = i;
+        if (!tu.natural)
+            std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
+                if (k == KIND_COLS && D[a].lgc != D[c].lgc) return D[a].lgc > D[c].lgc;
+                return (long)D[a].nu * D[a].nphi > (long)D[c].nu * D[c].nphi;
+            });
         const size_t start = q.size();
         for (int d : order)
             for (int j = 0; j < (*counts[k])[d]; j++) q.push_back(make_int2(d, j));
