@@ -46,7 +46,7 @@ constexpr int fx_minb(int threads, size_t smem) { return threads > 512 || 2 * sm
 // forward call, us: none 173.5, 2: 171.5, 3: 171.6, 4: 170.7; more spill)
 constexpr int FX_AHEAD = 4;
 
-// OR / maximum over one transform's NT threads (whole warps, or 8 or 16 lanes) into a shared word, zero before
+// OR / maximum / sum over one transform's NT threads (whole warps, or 8 or 16 lanes) into a shared word, zero before
 template <int NT>
 __device__ __forceinline__ void fx_or_into(unsigned f, unsigned* word)
 {
@@ -68,6 +68,18 @@ __device__ __forceinline__ void fx_max_into(unsigned f, unsigned* word)
         for (int o = NT / 2; o > 0; o >>= 1) f = max(f, __shfl_xor_sync(0xffffffffu, f, o));
     }
     if ((threadIdx.x & (NT < 32 ? NT - 1 : 31)) == 0) atomicMax(word, f);
+}
+
+template <int NT>
+__device__ __forceinline__ void fx_add_into(int f, int* word)
+{
+    if constexpr (NT >= 32) {
+        f = __reduce_add_sync(0xffffffffu, f);
+    } else {
+#pragma unroll
+        for (int o = NT / 2; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+    }
+    if ((threadIdx.x & (NT < 32 ? NT - 1 : 31)) == 0) atomicAdd(word, f);
 }
 
 __device__ __forceinline__ fx2 fx_ldg(const fx2* p)
@@ -207,11 +219,13 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
     constexpr int N = 1 << LG, NT = N / 8, SL = FxR2C<LG, BWD>::SL;
     extern __shared__ __align__(128) unsigned char smraw[];
     __shared__ unsigned nrm[SL][5];
-    __shared__ double2 level[SL];
+    __shared__ int level[SL][2];  // the rows' means, 2^29 at the exponent of the largest value
     unsigned char* const area = smraw + ((128 - (sg_smem_u32(smraw) & 127)) & 127);
     const int slot = threadIdx.x / NT, t = threadIdx.x % NT;
     fx2* const sm = reinterpret_cast<fx2*>(area) + (size_t)slot * (N + N / 16 + 1);
     if (t < 5) nrm[slot][t] = 0;
+    if (t < 2) level[slot][t] = 0;
+    __syncthreads();
     const int u = blockIdx.x * SL + slot, rows = BWD ? nu : nu / 2;
     const bool live = u < rows;
     const int i0 = BWD ? (live ? u : 0) : 2 * (live ? u : 0);
@@ -231,30 +245,45 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
     unsigned h = 0;
 #pragma unroll
     for (int e = 0; e < 8; e++) h = max(h, max(fx_abshi(z[e].x), fx_abshi(z[e].y)));
-    if (t == 0) level[slot] = z[0];
-    __syncthreads();
     fx_max_into<NT>(h, &nrm[slot][3]);
     __syncthreads();
     h = nrm[slot][3];
     const int F = fx_field(h);
     int E = fx_block_exp(h, F);
-    // each row less its first value (exact in fixed point, and added to the
-    // DC mode below), at the exponent of what is left: a disk's axisymmetric
-    // part would otherwise set the exponent its other modes are rounded at
-    const fx2 c{fx_from_double(level[slot].x, F), fx_from_double(level[slot].y, F)};
+    // Each row less its mean, at the exponent of what is left: a disk's
+    // axisymmetric part would otherwise set the exponent its other modes are
+    // rounded at.  The mean is formed from the values' high words (31 bits, an
+    // exact double), taken off exactly and added to the DC mode below, which
+    // holds next to nothing else: whatever the row, its sum takes one rounding.
+    // (Taking off the first value instead left the DC mode of a row with a peak
+    // there as the difference of two numbers N times as large: 1e-13 of it, and
+    // 1e-15 of the row in all other modes, at 4096 points.)
     fx2 v[8];
+    int mx = 0, my = 0;
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        v[e] = fx2{fx_from_double(z[e].x, F), fx_from_double(z[e].y, F)};
+        mx += fx_h(v[e].x);
+        my += fx_h(v[e].y);
+    }
+    constexpr int MS = LG - 3;  // the sum of the threads' eighths: 8 high words of the mean
+    fx_add_into<NT>((mx + (1 << MS >> 1)) >> MS, &level[slot][0]);
+    fx_add_into<NT>((my + (1 << MS >> 1)) >> MS, &level[slot][1]);
+    __syncthreads();
+    const fx2 c{(long long)level[slot][0] << 29, (long long)level[slot][1] << 29};
     unsigned g = 0;
 #pragma unroll
     for (int e = 0; e < 8; e++) {
-        v[e] = fx2{fx_from_double(z[e].x, F) - c.x, fx_from_double(z[e].y, F) - c.y};
+        v[e] = fx_sub(v[e], c);
         g |= fx_fold(v[e]);
     }
     fx_or_into<NT>(g, &nrm[slot][4]);
     __syncthreads();
     const int up = FX_T - fx_bits(nrm[slot][4]);
+    // (where the rest needs a bit more than the row had, the mean stays in)
 #pragma unroll
-    for (int e = 0; e < 8; e++) v[e] = up >= 0 ? fx2{v[e].x << up, v[e].y << up} : fx2{v[e].x >> 1, v[e].y >> 1};
-    E -= max(up, -1);
+    for (int e = 0; e < 8; e++) v[e] = up >= 0 ? fx2{v[e].x << up, v[e].y << up} : fx_add(v[e], c);
+    E -= max(up, 0);
     fx_fft<LG, -1>(v, sm, nrm[slot], t, tw, E);
     // X_a = (Z + conj Z[N - m]) / 2, X_b = (Z - conj Z[N - m]) / 2i
 #pragma unroll
@@ -276,9 +305,11 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
         }
         xa[e] = fx_out(p, E, safe);
         xb[e] = fx_out(q, E, safe);
-        if (e == 0 && t == 0) {
-            xa[0].x += N * level[slot].x;
-            xb[0].x += N * level[slot].y;
+        if (e == 0 && t == 0 && fx_bits(nrm[slot][4]) <= FX_T) {
+            const unsigned top = nrm[slot][3];
+            const int EM = fx_block_exp(top, fx_field(top)) + LG;
+            xa[0].x += fx_to_double_any((long long)level[slot][0] << 29, EM);
+            xb[0].x += fx_to_double_any((long long)level[slot][1] << 29, EM);
         }
     }
     const uint64_t keep = sg_policy_evict_last();  // the column pass reads the spectra from L2
