@@ -213,7 +213,10 @@ sg_status sg_plan_create(sg_plan** out, int N_u, int N_phi, double u_min, double
  * scratch of 6 N_u N_phi values.
  * Allocates and frees FP64 scratch for the spectra; radial_edges = 1 also
  * allocates the plan's edge tables, 2 (N_phi/2 + 1)(2 N_u + 1) values of
- * the working dtype.  Any other error than SG_ERR_TIMEOUT (SG_ERR_ALLOC,
+ * the working dtype.  SG_F32X2 plans allocate what their passes need the first
+ * time they are built for them (and when loaded): the fixed-point spectra,
+ * 32 (N_phi/2 + 1)(N_u + 2) bytes, or three double-float working fields.
+ * Any other error than SG_ERR_TIMEOUT (SG_ERR_ALLOC,
  * SG_ERR_CUDA, also from the set-up of sg_forces_noalloc at the end) leaves
  * the plan unbuilt: SG_ERR_NOT_BUILT until a build succeeds.
  */

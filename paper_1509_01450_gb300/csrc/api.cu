@@ -181,10 +181,9 @@ sg_status sg_plan_create(sg_plan** out, int nu, int nphi, double u_min, double d
         (st = dev_alloc(p, (void**)&p->keff, (size_t)2 * (2 * nu - 1) * nphi * sizeof(double))) ||
         // the fixed-point passes' tables, where either direction has such transforms
         (dtype != SG_F32 && (nphi >= 64 || nu >= 32) && (st = dev_alloc(p, &p->twx, fx_twiddle_bytes()))) ||
-        (dtype != SG_F32 && nu >= 32 &&
-         ((st = dev_alloc(p, &p->kfr, nk * 16)) || (st = dev_alloc(p, &p->kfp, nk * 16)))) ||
-        (dtype == SG_F32X2 && ((st = dev_alloc(p, &p->xf, (size_t)3 * nu * nphi * sizeof(dfloat))) ||
-                               (st = dev_alloc(p, &p->xw, (size_t)2 * nphi * sizeof(dfloat)))))) {
+        // (a compensated plan's buffers for one path or the other come with its build or file: path_buffers)
+        (dtype == SG_F64 && nu >= 32 &&
+         ((st = dev_alloc(p, &p->kfr, nk * 16)) || (st = dev_alloc(p, &p->kfp, nk * 16))))) {
         free_plan(p);
         return st;
     }
@@ -274,6 +273,30 @@ sg_status sg_plan_set_wait_limit(sg_plan* p, double seconds)
     return SG_OK;
 }
 
+// A compensated plan whose rows and columns both have fixed-point passes runs
+// them on its FP64 fields directly (1024 x 2048, forward and adjoint: 856 ->
+// 344 us).  The edge and wedge updates between the passes read double-float
+// spectra and tables, so plans with them (updates) keep the double-float passes.
+static bool fx_double_path(const PlanView& v, bool updates) { return !updates && fx_rows_ok(v) && fx_cols_len(v); }
+
+// What a compensated plan needs for its path, where it has not got it yet: the
+// fixed-point spectra, or the double-float working fields (2048 x 4096: 134
+// and 201 MB) and, with the wedge, the double-float wedge rows.
+static sg_status path_buffers(sg_plan* p, bool updates, bool wedge)
+{
+    if (p->dtype != SG_F32X2) return SG_OK;
+    const size_t nk = (size_t)(p->nphi / 2 + 1) * (p->nu + 2);
+    sg_status st = SG_OK;
+    if (fx_double_path(view(p), updates)) {
+        if ((!p->kfr && (st = dev_alloc(p, &p->kfr, nk * 16))) || (!p->kfp && (st = dev_alloc(p, &p->kfp, nk * 16))))
+            return st;
+    } else if (!p->xf && (st = dev_alloc(p, &p->xf, (size_t)3 * p->nu * p->nphi * sizeof(dfloat)))) {
+        return st;
+    }
+    if (wedge && !p->xw) st = dev_alloc(p, &p->xw, (size_t)2 * p->nphi * sizeof(dfloat));
+    return st;
+}
+
 // Plan file: a fixed header, then K̂_r, K̂_phi and the two weight rows in the
 // working dtype, exactly as they sit on the device.
 struct PlanFileHeader {
@@ -345,6 +368,10 @@ sg_status sg_plan_load(sg_plan** out, const char* path, cudaStream_t stream)
     if (!ok) {
         sg_plan_destroy(p);
         return SG_ERR_IO;
+    }
+    if ((st = path_buffers(p, false, false)) != SG_OK) {  // (files hold no edges and no wedge)
+        sg_plan_destroy(p);
+        return st;
     }
     if (cudaMemcpyAsync(p->kr, buf.data(), kb, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
         cudaMemcpyAsync(p->kp, buf.data() + kb, kb, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
@@ -472,6 +499,10 @@ sg_status sg_kernels_build(sg_plan* p, const sg_build_opts* opts, cudaStream_t s
             (!p->wtmp && (st = dev_alloc(p, &p->wtmp, (size_t)(nphi / 2) * sizeof(double2)))))
             return st;
     }
+    {
+        const sg_status st = path_buffers(p, edges || wedge, wedge != 0);
+        if (st) return st;
+    }
     int* flag = nullptr;
     double *nsr = nullptr, *nsp = nullptr, *wcells = nullptr;
     double2* W = nullptr;
@@ -569,15 +600,6 @@ static sg_status check_fields(const sg_plan* p, const void* a, const void* b, co
     return SG_OK;
 }
 
-// A compensated plan whose rows and columns both have fixed-point passes runs
-// them on its FP64 fields directly (1024 x 2048, forward and adjoint: 856 ->
-// 379 us).  The edge and wedge updates between the passes read double-float
-// spectra and tables, so plans with them keep the double-float passes.
-static bool fx_double_path(const sg_plan* p, const PlanView& v)
-{
-    return !p->edges && !p->wedge && fx_rows_ok(v) && fx_cols_ok(v);
-}
-
 // The passes on the plan's working type.  The compensated plans (SG_F32X2)
 // take and give FP64 fields; where they do not run on the fixed-point passes,
 // their inputs are split into double-float working fields first and the
@@ -589,7 +611,7 @@ static cudaError_t run_forward(sg_plan* p, PlanView v, const void* sigma, void* 
         return launch_forward<float>(v, (const float*)sigma, (float*)Fr, (float*)Fp, st, ev, direct);
     if (p->dtype == SG_F64)
         return launch_forward<double>(v, (const double*)sigma, (double*)Fr, (double*)Fp, st, ev, direct);
-    if (fx_double_path(p, v)) {
+    if (fx_double_path(v, p->edges || p->wedge)) {
         v.wdf = 1;
         return launch_forward<double>(v, (const double*)sigma, (double*)Fr, (double*)Fp, st, ev, direct);
     }
@@ -614,7 +636,7 @@ static cudaError_t run_backward(sg_plan* p, PlanView v, const void* gr, const vo
     if (p->dtype == SG_F32) return launch_backward<float>(v, (const float*)gr, (const float*)gp, (float*)gs, st, ev);
     if (p->dtype == SG_F64)
         return launch_backward<double>(v, (const double*)gr, (const double*)gp, (double*)gs, st, ev);
-    if (fx_double_path(p, v)) {
+    if (fx_double_path(v, p->edges || p->wedge)) {
         v.wdf = 1;
         return launch_backward<double>(v, (const double*)gr, (const double*)gp, (double*)gs, st, ev);
     }

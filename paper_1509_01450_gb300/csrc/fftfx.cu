@@ -27,7 +27,8 @@ bool fx_rows_ok(const PlanView& p)
     const FxKernels* k = p.twx ? fx_kernels(p.nphi) : nullptr;
     return k && p.nu % k->rows == 0 && fx_maps(p, k->rows);
 }
-bool fx_cols_ok(const PlanView& p) { return p.twx && p.kfr && fx_kernels(2 * p.nu); }
+bool fx_cols_len(const PlanView& p) { return p.twx && fx_kernels(2 * p.nu); }
+bool fx_cols_ok(const PlanView& p) { return p.kfr && p.kfp && fx_cols_len(p); }
 
 cudaError_t launch_fx_r2c(const PlanView& p, const double* x0, const double* x1, cudaStream_t st)
 {

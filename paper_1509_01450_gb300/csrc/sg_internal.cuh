@@ -33,7 +33,8 @@ struct sg_plan {
     void* kp;        // Khat_phi, same shape
     // FP64 and compensated plans: the fixed-point passes' tables (sg_fx.cuh):
     // both spectra as block fixed-point entries (null where 2 N_u has no
-    // fixed-point columns), the twiddles (null where neither direction has)
+    // fixed-point columns, or a compensated plan does not use them), the
+    // twiddles (null where neither direction has)
     void* kfr;
     void* kfp;
     void* twx;
@@ -48,7 +49,8 @@ struct sg_plan {
     // host-API staging (allocated on first sg_forces_host)
     // SG_F32X2: the double-float working fields of sigma, F_r, F_phi (or of
     // the adjoint's gF_r, gF_phi, gsigma) and of the wedge row's density and
-    // gradient (2 N_phi); the API's FP64 fields are converted into and out of them
+    // gradient (2 N_phi); the API's FP64 fields are converted into and out of
+    // them (null where the plan runs on the fixed-point passes; xw: no wedge)
     void* xf;
     void* xw;
     void* h_sigma;
@@ -219,10 +221,12 @@ cudaError_t launch_dft_c2r_adjoint(const PlanView& p, float* gs, cudaStream_t st
 cudaError_t launch_dft_tc_batch(const TcArgs* d_args, int n, int dir, int max_nu, cudaStream_t st);
 // fftfx.cu: the passes in 64-bit block fixed point (sg_fx.cuh), over FP64
 // fields and FP64 half spectra.  *_ok: the plan's rows (N_phi of 64 .. 4096,
-// their tensor maps made) or columns (2 N_u of 64 .. 4096) run on them;
+// their tensor maps made) or columns (2 N_u of 64 .. 4096: fx_cols_len, and the
+// fixed-point spectra there) run on them;
 // launch_fx_r2c's x1 and launch_fx_c2r's y1 are null for the forward R2C pass
 // and the adjoint C2R pass.
 bool fx_rows_ok(const PlanView& p);
+bool fx_cols_len(const PlanView& p);
 bool fx_cols_ok(const PlanView& p);
 cudaError_t launch_fx_r2c(const PlanView& p, const double* x0, const double* x1, cudaStream_t st);
 cudaError_t launch_fx_cols(const PlanView& p, bool adjoint, cudaStream_t st);
