@@ -1822,8 +1822,8 @@ struct RowUnit {
     static constexpr int GT = SMALL ? (NT < 32 ? 32 : NT) : LG <= 12 ? 256 : 512;  // threads per block
     static constexpr int TPG = GT / NT;              // paired transforms per block
     static constexpr int MINB = LG <= 12 ? SG_ROWS_MINB : 1;
-    // the area: the transforms' exchange areas (C2 elements), plus the 1 KB alignment slack
-    static constexpr size_t SMEM = (size_t)TPG * (N + N / 16 + 1) * 16 + 1024;
+    // the area: the transforms' exchange areas (C2 elements), plus the alignment slack
+    static constexpr size_t SMEM = (size_t)TPG * (N + N / 16 + 1) * 16 + 128;
 };
 
 // The half spectra of the real pairs packed in a paired transform: w holds
@@ -2343,8 +2343,7 @@ __host__ __device__ __forceinline__ size_t ring_cols_smem_bytes(int nu)
 template <int LG, bool BWD>
 __global__ void __launch_bounds__((1 << LG) / 16, 1)
     k_ring_cols(const float2* __restrict__ Kr, const float2* __restrict__ Kp, float2* __restrict__ out, int half,
-                const float2* __restrict__ tw, int* err, const __grid_constant__ CUtensorMap map, const float2* in,
-                int rows_layout)
+                const float2* __restrict__ tw, int* err, const __grid_constant__ CUtensorMap map)
 {
     constexpr int L = 1 << LG, nu = L / 2, NT = L / 16, KS = nu + 2;
     constexpr uint32_t ab = nu * (BWD ? 16 : 8), kb = KS * 8;
@@ -2365,12 +2364,8 @@ __global__ void __launch_bounds__((1 << LG) / 16, 1)
     const auto issue_column = [&](int m) {
         sg_fence_proxy_async();
         sg_mbar_expect_tx(&bar[0], ab);
-        SG_IF_OK(m < half && sg_smem_in(smraw, buf, ab), err, 321) {
-            if (rows_layout)
-                spec_load_column(buf, &map, m, nu / (BWD ? 2 : 4), &bar[0], drop);
-            else
-                sg_bulk_g2s_hint(buf, reinterpret_cast<const unsigned char*>(in) + (size_t)m * ab, ab, &bar[0], drop);
-        }
+        SG_IF_OK(m < half && sg_smem_in(smraw, buf, ab), err, 321)
+        spec_load_column(buf, &map, m, nu / (BWD ? 2 : 4), &bar[0], drop);
     };
     const auto issue_spectra = [&](int m) {
         sg_fence_proxy_async();
@@ -2411,8 +2406,7 @@ __global__ void __launch_bounds__((1 << LG) / 16, 1)
             float4* const P = reinterpret_cast<float4*>(out);
 #pragma unroll
             for (int e = 0; e < 8; e++) {  // crop to N_u rows
-                const int i = t + e * NT;
-                const size_t at = rows_layout ? spec_at(m, i ^ sw, half, 1) : (size_t)m * nu + i;
+                const size_t at = spec_at(m, (t + e * NT) ^ sw, half, 1);
                 SG_IF_OK(sg_in((long long)at, 1, (long long)half * nu), err, 323)
                 sg_st_hint(P + at, make_float4(f2_lo(w[e].x), f2_lo(w[e].y), f2_hi(w[e].x), f2_hi(w[e].y)), keep);
             }
@@ -2432,8 +2426,7 @@ __global__ void __launch_bounds__((1 << LG) / 16, 1)
             fft<16, +1, LG>(y, sm, L, LG, t, twd, isync);
 #pragma unroll
             for (int e = 0; e < 8; e++) {
-                const int i = t + e * NT;
-                const size_t at = rows_layout ? spec_at(m, i ^ (2 * sw), half, 2) : (size_t)m * nu + i;
+                const size_t at = spec_at(m, (t + e * NT) ^ (2 * sw), half, 2);
                 SG_IF_OK(sg_in((long long)at, 1, (long long)half * nu), err, 324)
                 sg_st_hint(out + at, y[e], keep);
             }
@@ -2465,8 +2458,7 @@ typedef void (*BwdColsFn)(const float2*, const float2*, const float2*, const flo
                           const float2*, int*, const float*, const float*, const float*, EdgeCoef<float>,
                           CUtensorMap, CUtensorMap, int, const float*, float2*);
 
-typedef void (*RingColsFn)(const float2*, const float2*, float2*, int, const float2*, int*, CUtensorMap, const float2*,
-                           int);
+typedef void (*RingColsFn)(const float2*, const float2*, float2*, int, const float2*, int*, CUtensorMap);
 
 typedef void (*RingR2CFn)(const float*, const float*, const float*, float2*, int, const float2*, int*);
 typedef void (*RingC2RFn)(const float4*, const float*, float*, float*, int, const float2*, int*);
@@ -2584,23 +2576,7 @@ static Shape shape_for(int n, int min_threads)
 template <typename K>
 static int persistent_grid(K kernel, int threads, size_t smem, int nblk, int sms)
 {
-    LaunchCache& c = launch_cache();
-    const auto key = std::make_tuple((const void*)kernel, current_device(), threads, smem);
-    int occ = 0;
-    {
-        std::lock_guard<std::mutex> lock(c.mu);
-        auto it = c.occ.find(key);
-        if (it != c.occ.end()) occ = it->second;
-    }
-    if (occ == 0) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem) != cudaSuccess || occ < 1) {
-            cudaGetLastError();
-            occ = 1;
-        }
-        std::lock_guard<std::mutex> lock(c.mu);
-        c.occ[key] = occ;
-    }
-    const int g = occ * (sms > 0 ? sms : 1);
+    const int g = resident_blocks(kernel, threads, smem, sms);
     return nblk < g ? nblk : g;
 }
 
@@ -2761,11 +2737,12 @@ static bool fixed_path(const PlanView& p, const FixedPassKernels*& fr, const Fix
 
 // The persistent column passes: one block per SM, each taking every grid-th
 // mode.  Not for at most one mode per SM, where k_fwd_cols copies the spectra
-// before the row pass ends (4096 x 32 forward: 21.0 against 22.6 us), and not
-// with edge tables, for which the buffer leaves no room.
+// before the row pass ends (4096 x 32 forward: 21.0 against 22.6 us), not with
+// edge tables, for which the buffer leaves no room, and on the row layout only
+// (tensor-core rows have fewer modes than the GPU has SMs).
 static bool ring_cols_fit(const PlanView& p, const FixedPassKernels* fc)
 {
-    return p.pairs && !p.edges && fc->ring_cols[0] && p.nphi / 2 > p.sms;
+    return p.pairs == 2 && !p.edges && fc->ring_cols[0] && p.nphi / 2 > p.sms;
 }
 // The persistent row passes, rows_per_unit rows each: not for at most one unit
 // per SM, which they would only delay, nor for the wedge's extra row.
@@ -2797,14 +2774,9 @@ static cudaError_t launch_ring_cols(const PlanView& p, RingColsFn k, bool adjoin
     const size_t smem = ring_cols_smem_bytes(p.nu);
     cudaError_t err = set_smem(k, smem, true);
     if (err != cudaSuccess) return err;
-    const int half = p.nphi / 2;
-    float2* const single = (float2*)p.wa;
-    float2* const pairs = (float2*)p.wb;
-    const CUtensorMap none{};
-    return launch_pdl(k, half < p.sms ? half : p.sms, 2 * p.nu / 16, smem, st, (const float2*)p.kr,
-                      (const float2*)p.kp, adjoint ? single : pairs, half, (const float2*)p.tw, p.err,
-                      p.pairs == 2 ? p.imaps[adjoint ? 0 : 1] : none, (const float2*)(adjoint ? pairs : single),
-                      p.pairs == 2);
+    return launch_pdl(k, p.sms, 2 * p.nu / 16, smem, st, (const float2*)p.kr, (const float2*)p.kp,
+                      (float2*)(adjoint ? p.wa : p.wb), p.nphi / 2, (const float2*)p.tw, p.err,
+                      p.imaps[adjoint ? 0 : 1]);
 }
 
 template <typename T>
