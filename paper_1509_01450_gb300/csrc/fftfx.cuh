@@ -46,7 +46,7 @@ constexpr int fx_minb(int threads, size_t smem) { return threads > 512 || 2 * sm
 // forward call, us: none 173.5, 2: 171.5, 3: 171.6, 4: 170.7; more spill)
 constexpr int FX_AHEAD = 4;
 
-// OR / maximum / sum over one transform's NT threads (whole warps, or 8 or 16 lanes) into a shared word, zero before
+// OR / maximum over one transform's NT threads (whole warps, or 8 or 16 lanes) into a shared word, zero before
 template <int NT>
 __device__ __forceinline__ void fx_or_into(unsigned f, unsigned* word)
 {
@@ -70,16 +70,37 @@ __device__ __forceinline__ void fx_max_into(unsigned f, unsigned* word)
     if ((threadIdx.x & (NT < 32 ? NT - 1 : 31)) == 0) atomicMax(word, f);
 }
 
-template <int NT>
-__device__ __forceinline__ void fx_add_into(int f, int* word)
+// the same of two values into two words, by two lanes at once
+struct FxOr {
+    static __device__ __forceinline__ unsigned warp(unsigned a) { return __reduce_or_sync(0xffffffffu, a); }
+    static __device__ __forceinline__ unsigned of(unsigned a, unsigned b) { return a | b; }
+    static __device__ __forceinline__ void into(unsigned* w, unsigned a) { atomicOr(w, a); }
+};
+struct FxMax {
+    static __device__ __forceinline__ unsigned warp(unsigned a) { return __reduce_max_sync(0xffffffffu, a); }
+    static __device__ __forceinline__ unsigned of(unsigned a, unsigned b) { return max(a, b); }
+    static __device__ __forceinline__ void into(unsigned* w, unsigned a) { atomicMax(w, a); }
+};
+struct FxSum {
+    static __device__ __forceinline__ unsigned warp(unsigned a) { return __reduce_add_sync(0xffffffffu, a); }
+    static __device__ __forceinline__ unsigned of(unsigned a, unsigned b) { return a + b; }
+    static __device__ __forceinline__ void into(unsigned* w, unsigned a) { atomicAdd(w, a); }
+};
+template <int NT, typename Op>
+__device__ __forceinline__ void fx_both_into(unsigned a, unsigned b, unsigned* words)
 {
     if constexpr (NT >= 32) {
-        f = __reduce_add_sync(0xffffffffu, f);
+        a = Op::warp(a);
+        b = Op::warp(b);
     } else {
 #pragma unroll
-        for (int o = NT / 2; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+        for (int o = NT / 2; o > 0; o >>= 1) {
+            a = Op::of(a, __shfl_xor_sync(0xffffffffu, a, o));
+            b = Op::of(b, __shfl_xor_sync(0xffffffffu, b, o));
+        }
     }
-    if ((threadIdx.x & (NT < 32 ? NT - 1 : 31)) == 0) atomicAdd(word, f);
+    const int lane = threadIdx.x & (NT < 32 ? NT - 1 : 31);
+    if (lane < 2) Op::into(words + lane, lane ? b : a);
 }
 
 __device__ __forceinline__ fx2 fx_ldg(const fx2* p)
@@ -196,6 +217,34 @@ __device__ __forceinline__ void fx_st256(double2* p, double2 a, double2 b, uint6
                  : "memory");
 }
 
+// The means of a pair of rows, each at the exponent of its row's largest value:
+// 31 bits, 2^29 sum, or the first value where that is within 2^-20 of it, so
+// that a constant row leaves nothing.
+struct FxLevel {
+    unsigned sum[2];
+    fx2 first;
+    static __device__ __forceinline__ long long pick(unsigned sum, long long first)
+    {
+        const long long m = (long long)(int)sum << 29;
+        return fx_fold(first - m) < 1u << (FX_T - 20 - 32) ? first : m;
+    }
+    __device__ __forceinline__ fx2 mean() const { return fx2{pick(sum[0], first.x), pick(sum[1], first.y)}; }
+};
+// the exponent above the rest that a row leaves (folded), -FX_BAD for none
+__device__ __forceinline__ int fx_rest_top(int E, unsigned folded)
+{
+    return folded || E == FX_BAD ? E + min(fx_bits(folded), FX_T) : -FX_BAD;
+}
+// a row's DC mode with the mean c that was taken off; largest, rest: its nrm words
+template <int LG>
+__device__ __forceinline__ double fx_with_mean(double dc, long long c, unsigned largest, unsigned rest)
+{
+    if (fx_bits(rest) > FX_T) return dc;
+    const int E = fx_block_exp(largest, fx_field(largest)) + LG;
+    const long long hi = c & ~((1ll << 29) - 1);  // exact as a double
+    return dc + fx_to_double_any(c - hi, E) + fx_to_double_any(hi, E);
+}
+
 // ---------------------------------------------------------------------------
 // P1 / P1b: one complex transform of two real sequences per slot, split into
 // their half spectra.  Forward: rows 2p, 2p + 1 of sigma (x0), both halves to
@@ -218,13 +267,13 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
 {
     constexpr int N = 1 << LG, NT = N / 8, SL = FxR2C<LG, BWD>::SL;
     extern __shared__ __align__(128) unsigned char smraw[];
-    __shared__ unsigned nrm[SL][5];
-    __shared__ int level[SL][2];  // the rows' means, 2^29 at the exponent of the largest value
+    __shared__ unsigned nrm[SL][7];  // the transform's three, the rows' largest values and those of their rests
+    __shared__ FxLevel level[SL];
     unsigned char* const area = smraw + ((128 - (sg_smem_u32(smraw) & 127)) & 127);
     const int slot = threadIdx.x / NT, t = threadIdx.x % NT;
     fx2* const sm = reinterpret_cast<fx2*>(area) + (size_t)slot * (N + N / 16 + 1);
-    if (t < 5) nrm[slot][t] = 0;
-    if (t < 2) level[slot][t] = 0;
+    if (t < 7) nrm[slot][t] = 0;
+    if (t < 2) level[slot].sum[t] = 0;
     __syncthreads();
     const int u = blockIdx.x * SL + slot, rows = BWD ? nu : nu / 2;
     const bool live = u < rows;
@@ -242,48 +291,63 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
 #pragma unroll
         for (int e = 0; e < 8; e++) z[e] = double2{z[e].x * w0, z[e].y * w1};
     }
-    unsigned h = 0;
-#pragma unroll
-    for (int e = 0; e < 8; e++) h = max(h, max(fx_abshi(z[e].x), fx_abshi(z[e].y)));
-    fx_max_into<NT>(h, &nrm[slot][3]);
-    __syncthreads();
-    h = nrm[slot][3];
-    const int F = fx_field(h);
-    int E = fx_block_exp(h, F);
-    // Each row less its mean, at the exponent of what is left: a disk's
-    // axisymmetric part would otherwise set the exponent its other modes are
-    // rounded at.  The mean is formed from the values' high words (31 bits, an
-    // exact double), taken off exactly and added to the DC mode below, which
-    // holds next to nothing else: whatever the row, its sum takes one rounding.
-    // (Taking off the first value instead left the DC mode of a row with a peak
-    // there as the difference of two numbers N times as large: 1e-13 of it, and
-    // 1e-15 of the row in all other modes, at 4096 points.)
-    fx2 v[8];
-    int mx = 0, my = 0;
+    unsigned h0 = 0, h1 = 0;
 #pragma unroll
     for (int e = 0; e < 8; e++) {
-        v[e] = fx2{fx_from_double(z[e].x, F), fx_from_double(z[e].y, F)};
-        mx += fx_h(v[e].x);
-        my += fx_h(v[e].y);
+        h0 = max(h0, fx_abshi(z[e].x));
+        h1 = max(h1, fx_abshi(z[e].y));
     }
-    constexpr int MS = LG - 3;  // the sum of the threads' eighths: 8 high words of the mean
-    fx_add_into<NT>((mx + (1 << MS >> 1)) >> MS, &level[slot][0]);
-    fx_add_into<NT>((my + (1 << MS >> 1)) >> MS, &level[slot][1]);
+    fx_both_into<NT, FxMax>(h0, h1, &nrm[slot][3]);
     __syncthreads();
-    const fx2 c{(long long)level[slot][0] << 29, (long long)level[slot][1] << 29};
-    unsigned g = 0;
+    // Each row less its mean, and both at the exponent of what is left: a
+    // disk's axisymmetric part would otherwise set the exponent that its other
+    // modes are rounded at, and an axisymmetric row that of the weaker row that
+    // shares its transform (1e-12 of a row of 1e-6 beside a constant 1).  The
+    // mean is taken off exactly and added to the DC mode below, which holds
+    // next to nothing else: whatever the row, its sum takes one rounding.
+    // (Taking off the first value left the DC mode of a row with a peak there
+    // as the difference of two numbers N times as large: 1e-13 of it, and 1e-15
+    // of the row in all other modes, at 4096 points.)
+    const int F0 = fx_field(nrm[slot][3]), F1 = fx_field(nrm[slot][4]);
+    fx2 v[8];
+    int m0 = 0, m1 = 0;
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        v[e] = fx2{fx_from_double(z[e].x, F0), fx_from_double(z[e].y, F1)};
+        m0 += fx_h(v[e].x);
+        m1 += fx_h(v[e].y);
+    }
+    constexpr int MS = LG - 3;  // the sum of the threads' eighths: 8 high words of the mean, below 2^31
+    fx_both_into<NT, FxSum>((m0 + (1 << MS >> 1)) >> MS, (m1 + (1 << MS >> 1)) >> MS, level[slot].sum);
+    if (t == 0) level[slot].first = v[0];
+    __syncthreads();
+    const fx2 c = level[slot].mean();
+    unsigned g0 = 0, g1 = 0;
 #pragma unroll
     for (int e = 0; e < 8; e++) {
         v[e] = fx_sub(v[e], c);
-        g |= fx_fold(v[e]);
+        g0 |= fx_fold(v[e].x);
+        g1 |= fx_fold(v[e].y);
     }
-    fx_or_into<NT>(g, &nrm[slot][4]);
+    fx_both_into<NT, FxOr>(g0, g1, &nrm[slot][5]);
     __syncthreads();
-    const int up = FX_T - fx_bits(nrm[slot][4]);
-    // (where the rest needs a bit more than the row had, the mean stays in)
+    g0 = nrm[slot][5];
+    g1 = nrm[slot][6];
+    if (fx_bits(g0 | g1) > FX_T) {  // a rest that needs a bit more than its row had keeps the mean
+        const fx2 k{fx_bits(g0) > FX_T ? c.x : 0, fx_bits(g1) > FX_T ? c.y : 0};
 #pragma unroll
-    for (int e = 0; e < 8; e++) v[e] = up >= 0 ? fx2{v[e].x << up, v[e].y << up} : fx_add(v[e], c);
-    E -= max(up, 0);
+        for (int e = 0; e < 8; e++) v[e] = fx_add(v[e], k);
+    }
+    const int E0 = fx_block_exp(nrm[slot][3], F0), E1 = fx_block_exp(nrm[slot][4], F1);
+    const int top = max(fx_rest_top(E0, g0), fx_rest_top(E1, g1));
+    int E = top == -FX_BAD ? E0 : top - FX_T;
+    const int l0 = min(max(E0 - E, 0), 63), l1 = min(max(E1 - E, 0), 63);
+#pragma unroll
+    for (int e = 0; e < 8; e++) v[e] = fx2{v[e].x << l0, v[e].y << l1};
+    if (E > min(E0, E1)) {  // the weaker row gives way
+#pragma unroll
+        for (int e = 0; e < 8; e++) v[e] = fx2{fx_shift(v[e].x, max(E - E0, 0)), fx_shift(v[e].y, max(E - E1, 0))};
+    }
     fx_fft<LG, -1>(v, sm, nrm[slot], t, tw, E);
     // X_a = (Z + conj Z[N - m]) / 2, X_b = (Z - conj Z[N - m]) / 2i
 #pragma unroll
@@ -305,11 +369,10 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
         }
         xa[e] = fx_out(p, E, safe);
         xb[e] = fx_out(q, E, safe);
-        if (e == 0 && t == 0 && fx_bits(nrm[slot][4]) <= FX_T) {
-            const unsigned top = nrm[slot][3];
-            const int EM = fx_block_exp(top, fx_field(top)) + LG;
-            xa[0].x += fx_to_double_any((long long)level[slot][0] << 29, EM);
-            xb[0].x += fx_to_double_any((long long)level[slot][1] << 29, EM);
+        if (e == 0 && t == 0) {
+            const fx2 c = level[slot].mean();
+            xa[0].x = fx_with_mean<LG>(xa[0].x, c.x, nrm[slot][3], nrm[slot][5]);
+            xb[0].x = fx_with_mean<LG>(xb[0].x, c.y, nrm[slot][4], nrm[slot][6]);
         }
     }
     const uint64_t keep = sg_policy_evict_last();  // the column pass reads the spectra from L2
