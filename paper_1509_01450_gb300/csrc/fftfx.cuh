@@ -670,9 +670,10 @@ __global__ void __launch_bounds__(FxCols<LG>::THREADS, FxCols<LG>::MINB)
 // rows Z = S_i0 + i S_i1, gsigma of i0, i0 + 1 = Re, Im.  The rows' modes
 // arrive by 2-D tensor copies as S[m RB + r] (B, then C), each slot turns its
 // own modes into fixed point in place (once, not once per use), and the
-// exchange areas then lie over the stage.  The DC terms stay out of the
-// transform and are added to its rows: a disk's axisymmetric part would
-// otherwise set the exponent that its other modes are rounded at.
+// exchange areas then lie over the stage.  The DC and Nyquist terms stay out of
+// the transform and are added to its rows: a disk's axisymmetric part, and what
+// the column pass's rounding of it leaves in the Nyquist mode that it is packed
+// with, would otherwise set the exponent that its other modes are rounded at.
 // ---------------------------------------------------------------------------
 template <int LG, bool BWD>
 struct FxC2R {
@@ -718,7 +719,11 @@ __global__ void __launch_bounds__(FxC2R<LG, BWD>::THREADS, FxC2R<LG, BWD>::MINB)
     // this slot's two half spectra: element m at S0[m RB], S1[m RB]
     double2* const S0 = reinterpret_cast<double2*>(area) + (BWD ? 2 * slot : slot);
     double2* const S1 = BWD ? S0 + 1 : S0 + (size_t)half * RB;
-    const double dc0 = S0[0].x, dc1 = BWD ? S1[0].x : 0.0;  // (the azimuthal force has none)
+    // (DC, Nyquist), which this thread's places take as one number: N / 8 is even
+    // (forward: the azimuthal force has neither)
+    const double2 ends0 = S0[0], ends1 = BWD ? S1[0] : double2{0.0, 0.0};
+    const double end0 = t & 1 ? ends0.x - ends0.y : ends0.x + ends0.y;
+    const double end1 = t & 1 ? ends1.x - ends1.y : ends1.x + ends1.y;
     int E;
     {
         double2 a[4], b[4];
@@ -727,7 +732,7 @@ __global__ void __launch_bounds__(FxC2R<LG, BWD>::THREADS, FxC2R<LG, BWD>::MINB)
         for (int e = 0; e < 4; e++) {
             a[e] = S0[(t + e * NT) * RB];
             b[e] = S1[(t + e * NT) * RB];
-            if (e == 0 && t == 0) a[0].x = b[0].x = 0.0;
+            if (e == 0 && t == 0) a[0] = b[0] = double2{0.0, 0.0};
             h = max(h, max(max(fx_abshi(a[e].x), fx_abshi(a[e].y)), max(fx_abshi(b[e].x), fx_abshi(b[e].y))));
         }
         fx_max_into<NT>(h, &nrm[slot][3]);
@@ -747,14 +752,8 @@ __global__ void __launch_bounds__(FxC2R<LG, BWD>::THREADS, FxC2R<LG, BWD>::MINB)
     for (int e = 0; e < 8; e++) {
         const int n = t + e * NT, mo = e < 4 ? n : (n == half ? 0 : N - n);
         const fx2 a = reinterpret_cast<const fx2*>(S0)[mo * RB], b = reinterpret_cast<const fx2*>(S1)[mo * RB];
-        if (e == 0 && t == 0)
-            v[e] = fx2{0, 0};  // DC, added below
-        else if (e == 4 && t == 0)
-            v[e] = fx2{a.y, BWD ? b.y : 0};  // Nyquist
-        else if (e < 4)
-            v[e] = fx2{a.x - b.y, a.y + b.x};  // a + i b
-        else
-            v[e] = fx2{a.x + b.y, b.x - a.y};  // conj a + i conj b
+        v[e] = e < 4 ? fx2{a.x - b.y, a.y + b.x}   // a + i b
+                     : fx2{a.x + b.y, b.x - a.y};  // conj a + i conj b
     }
     __syncthreads();  // the exchange areas lie over the stage
     fx_fft<LG, +1>(v, sm, nrm[slot], t, tw, E);
@@ -765,8 +764,8 @@ __global__ void __launch_bounds__(FxC2R<LG, BWD>::THREADS, FxC2R<LG, BWD>::MINB)
 #pragma unroll
     for (int e = 0; e < 8; e++) {
         z[e] = fx_out(v[e], E, safe);
-        z[e].x += dc0;
-        if (BWD) z[e].y += dc1;
+        z[e].x += end0;
+        if (BWD) z[e].y += end1;
     }
     if (fx_weighted(w0, w1)) {
         asm volatile("" ::: "memory");  // stays a branch
