@@ -314,8 +314,8 @@ __global__ void __launch_bounds__(FxR2C<LG, BWD>::THREADS, FxR2C<LG, BWD>::MINB)
 #pragma unroll
     for (int e = 0; e < 8; e++) {
         v[e] = fx2{fx_from_double(z[e].x, F0), fx_from_double(z[e].y, F1)};
-        m0 += fx_h(v[e].x);
-        m1 += fx_h(v[e].y);
+        m0 += (int)(v[e].x >> 32);
+        m1 += (int)(v[e].y >> 32);
     }
     constexpr int MS = LG - 3;  // the sum of the threads' eighths: 8 high words of the mean, below 2^31
     fx_both_into<NT, FxSum>((m0 + (1 << MS >> 1)) >> MS, (m1 + (1 << MS >> 1)) >> MS, level[slot].sum);
@@ -694,6 +694,7 @@ __global__ void __launch_bounds__(FxC2R<LG, BWD>::THREADS, FxC2R<LG, BWD>::MINB)
     extern __shared__ __align__(128) unsigned char smraw[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ unsigned nrm[SL][4];
+    __shared__ double2 ends[SL][2];
     unsigned char* const area = smraw + ((128 - (sg_smem_u32(smraw) & 127)) & 127);
     const int slot = threadIdx.x / NT, t = threadIdx.x % NT;
     fx2* const sm = reinterpret_cast<fx2*>(area) + (size_t)slot * (N + N / 16 + 1);
@@ -719,11 +720,10 @@ __global__ void __launch_bounds__(FxC2R<LG, BWD>::THREADS, FxC2R<LG, BWD>::MINB)
     // this slot's two half spectra: element m at S0[m RB], S1[m RB]
     double2* const S0 = reinterpret_cast<double2*>(area) + (BWD ? 2 * slot : slot);
     double2* const S1 = BWD ? S0 + 1 : S0 + (size_t)half * RB;
-    // (DC, Nyquist), which this thread's places take as one number: N / 8 is even
-    // (forward: the azimuthal force has neither)
-    const double2 ends0 = S0[0], ends1 = BWD ? S1[0] : double2{0.0, 0.0};
-    const double end0 = t & 1 ? ends0.x - ends0.y : ends0.x + ends0.y;
-    const double end1 = t & 1 ? ends1.x - ends1.y : ends1.x + ends1.y;
+    if (t < 2) {  // DC +- Nyquist, which even and odd places take as one number (the azimuthal force has neither)
+        const double2 a = S0[0], b = BWD ? S1[0] : double2{0.0, 0.0};
+        ends[slot][t] = t ? double2{a.x - a.y, b.x - b.y} : double2{a.x + a.y, b.x + b.y};
+    }
     int E;
     {
         double2 a[4], b[4];
@@ -760,12 +760,13 @@ __global__ void __launch_bounds__(FxC2R<LG, BWD>::THREADS, FxC2R<LG, BWD>::MINB)
     const bool safe = fx_exp_safe(E);
     double* const o0 = y0 + (size_t)i0 * N + t;
     double* const o1 = BWD ? y0 + (size_t)(i0 + 1) * N + t : y1 + (size_t)i0 * N + t;
+    const double2 end = ends[slot][t & 1];  // N / 8 is even: the parity of all its places
     double2 z[8];
 #pragma unroll
     for (int e = 0; e < 8; e++) {
         z[e] = fx_out(v[e], E, safe);
-        z[e].x += end0;
-        if (BWD) z[e].y += end1;
+        z[e].x += end.x;
+        if (BWD) z[e].y += end.y;
     }
     if (fx_weighted(w0, w1)) {
         asm volatile("" ::: "memory");  // stays a branch
