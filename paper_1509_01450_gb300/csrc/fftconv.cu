@@ -34,8 +34,9 @@
 //
 // Plans with one-sided radial edge slopes add a rank-4 update per mode
 // after P2 (inside P2 for FP32 with 16 points per thread) and its transpose
-// after P2b.  FP32 transforms of 2^8 .. 2^13 points run instances with the
-// length fixed at compile time, compiled in fftconv_lg<LG>.cu.
+// after P2b.  FP32 rows of 2^8 .. 2^13 points and columns of 2^6 .. 2^13 run
+// instances with the length fixed at compile time, compiled in
+// fftconv_lg<LG>.cu.
 #include <mutex>
 
 #include "sg_internal.cuh"
@@ -91,8 +92,8 @@ struct EdgeCoef {
 };
 
 // The origin wedge's update fused into the forward column pass: the wedge
-// row's phi-spectrum per mode (swh, written by k_wedge_dft before the row
-// pass) and the plan's wedge tables [4][N_phi/2 + 1][N_u] (Wr, Wphi, Vr, Vphi).
+// row's phi-spectrum per mode (swh, written by a block of the fixed-length row
+// pass, else by k_wedge_dft before the row pass) and the plan's wedge tables [4][N_phi/2 + 1][N_u] (Wr, Wphi, Vr, Vphi).
 template <typename T>
 struct WedgeArgs {
     const typename CX<T>::t* swh;
@@ -2096,7 +2097,7 @@ __device__ __forceinline__ void rows_c2r_math(const float4* S4, const float (&wt
 }
 
 // One unit of the row C2R pass (rows u R .. u R + R - 1), shared like
-// rows_r2c_unit; map: the tensor map in kernel-parameter or global memory.
+// rows_r2c_unit; in: the spectra in the row layout (forward: pairs).
 template <int LG, bool BWD, bool PDL, bool SMALL = false>
 __device__ __forceinline__ bool rows_c2r_unit(const float4* in, const float* __restrict__ wrow,
                                               float* __restrict__ y0, float* __restrict__ y1, int nu,
@@ -2440,7 +2441,7 @@ __global__ void __launch_bounds__((1 << LG) / 16, 1)
 // (fftconv_lg<LG>.cu, which includes this file for its kernels only) and
 // reached through fixed_pass_kernels().  A plan whose row length N_phi and
 // column length 2 N_u both have instances runs all its passes on them, with
-// the column spectra in the pair layout; other plans take the run-time
+// the column spectra in the row layout; other plans take the run-time
 // instances and separate B, C buffers.  Row blocks are 256 threads up to
 // 4096 points (several slots below), one 512-thread transform beyond;
 // column blocks are one transform of 2 N_u / 16 threads.
@@ -2711,14 +2712,14 @@ static cudaError_t launch_edges(const PlanView& p, bool adjoint, cudaStream_t st
 
 // The fixed-length instances of both transform lengths, when every pass of
 // the plan can run on them: FP32, N_phi of 256 .. 8192 and 2 N_u of 64 .. 8192
-// points, the pair layout's tensor maps made, N_u a multiple of the small row
+// points, the row layout's tensor maps made, N_u a multiple of the small row
 // blocks (and then of the others where pick takes those: N_u is a power of
-// two).  The passes then keep the column spectra in the pair layout.  Columns
+// two).  The passes then keep the column spectra in the row layout.  Columns
 // of 64 and 128 points came in for the rows' sake: the three passes of 64 x
 // 1024, launched apart, 27.6 -> 21.2 us (adjoint 30.4 -> 22.3), 32 x 8192
 // chained 36.2 -> 29.0.  Tensor-core rows
-// (short_dft) read and write that layout at any of their lengths, so with them
-// only the columns have to qualify (fr null where the rows have no instances):
+// (short_dft) read and write pairs of contiguous columns at any of their
+// lengths, so with them only the columns have to qualify (fr null where the rows have no instances):
 // a 4096 x 32 forward call, with the row passes chained by programmatic
 // launch as well, 29.2 -> 21.0 us.
 template <typename T>

@@ -9,7 +9,7 @@
 // points is held by N / 8 threads, 8 points each (32 registers); exchanges go
 // through 16-byte elements in shared memory, padded as sg_pad.  Each thread's
 // twiddles come from tables laid out by pass (fx_tw_base), read through L1:
-// their 61 bits would cost more to form by products.
+// their 62 bits would cost more to form by products.
 //
 // What bounds them: the integer pipes (a complex product is twelve wide
 // multiply-adds and some fifteen additions and moves), and before that the

@@ -30,7 +30,8 @@ LIB_PATH = os.path.join(_HERE, "libsgdisk_checked.so" if _VARIANT == "checked" e
  SG_ERR_BOUNDS) = range(9)
 SG_F32, SG_F64, SG_F32X2 = 0, 1, 2
 # plan precisions by name: FP32, FP64, and the compensated FP32 plans
-# (double-float passes on the FP32 pipes; fields FP64 like SG_F64)
+# (fields FP64 like SG_F64, kernel spectra in two floats; the passes in 64-bit
+# fixed point, or in double-floats on the FP32 pipes where those do not apply)
 PRECISIONS = {"float32": SG_F32, "f32": SG_F32, "torch.float32": SG_F32, "float64": SG_F64, "f64": SG_F64,
               "torch.float64": SG_F64, "float32x2": SG_F32X2, "f32x2": SG_F32X2, "compensated": SG_F32X2}
 
