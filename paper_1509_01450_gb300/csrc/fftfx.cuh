@@ -19,7 +19,7 @@
 // instructions.  Here the radix-8 passes of a kernel are one loop, and the
 // column kernels' three transforms share it (inverses as conj FFT conj).
 // Measured at 1024 x 2048, the FP64 pipe's kernels -> these, us: R2C rows 105
-// -> 31, columns 486 -> 99, C2R rows 195 -> 52; a forward call 781 -> 171.
+// -> 32, columns 486 -> 98, C2R rows 195 -> 51; a forward call 781 -> 169.
 // Products that shifted their sums into place, and whose digits' products the
 // compiler widened to 64 x 64 bits, took 32, 111, 55 and 188.
 // Error of F_phi on a smooth disk of 256 x 512 against an 80-bit evaluation:
