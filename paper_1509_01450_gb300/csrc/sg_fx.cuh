@@ -91,6 +91,12 @@ FXHD long long fx_rmul(long long a)
     return a - fx_join(fx_wide(ah, rh, FX_HI), fx_wide(al, rh, fx_wide(ah, rl, FX_MID)));
 }
 
+// (a + b) / 2 and (a - b) / 2 without the sum's extra bit, off by half a unit at
+// most and by nothing on average: the sum's halves are rounded one down, one
+// up, the difference's both down
+FXHD long long fx_half_sum(long long a, long long b) { return (a >> 1) + (b >> 1) + (b & 1); }
+FXHD long long fx_half_diff(long long a, long long b) { return (a >> 1) - (b >> 1); }
+
 FXHD fx2 fx_add(fx2 a, fx2 b) { return fx2{a.x + b.x, a.y + b.y}; }
 FXHD fx2 fx_sub(fx2 a, fx2 b) { return fx2{a.x - b.x, a.y - b.y}; }
 // x + DIR i d
