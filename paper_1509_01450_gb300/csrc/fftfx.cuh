@@ -459,13 +459,17 @@ __device__ __forceinline__ fx2 fx_product(fx2 a, fx2 w, int dE, unsigned& top)
     top = max(top, (unsigned)(fx_bits(fx_fold(p)) + 64 - dE));
     return p;
 }
-// a product at the block's exponent: shift = bits above FX_T of the largest
+// a product at the block's exponent: shift = bits above FX_T of the largest.
+// Ties (one product in four at a shift of 1) go up at even frequencies and down
+// at odd ones (t's parity: N / 8 is even): the bias of one sign that all going up
+// leaves would add up in row 0 (2.5e-15 of F_r's rms at 2048 rows), this one's
+// sum lies N_u rows on, where the column is cropped.
 template <int NT, bool SECOND>
 __device__ __forceinline__ fx2 fx_align(fx2 p, const FxSpecRows& K, int t, int e, int shift)
 {
     const int2* w = reinterpret_cast<const int2*>((SECOND ? K.k2 : K.k1) + fx_spec_index<NT>(t, e));
     const int d = ((__ldg(&w[0].x) & 7) | (__ldg(&w[1].x) & 7) << 3) + shift;
-    return fx2{fx_shift(p.x, d), fx_shift(p.y, d)};
+    return fx2{fx_shift(p.x, d, t & 1), fx_shift(p.y, d, t & 1)};
 }
 
 template <int LG>

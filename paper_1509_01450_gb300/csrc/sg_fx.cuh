@@ -185,11 +185,12 @@ FXHD unsigned fx_fold(const fx2 (&v)[8])
 // bits of the block's largest component from the OR of fx_fold
 FXHD int fx_bits(unsigned folded) { return 64 - fx_clz32(folded); }
 
-// x 2^-d, rounded, or x 2^-d for d < 0; |x| <= 2^62, so that d >= 63 gives 0
-FXHD long long fx_shift(long long x, int d)
+// x 2^-d, rounded, or x 2^-d for d < 0; |x| <= 2^62, so that d >= 63 gives 0;
+// a tie goes up, or down for odd = 1
+FXHD long long fx_shift(long long x, int d, int odd = 0)
 {
     const int l = d > 0 ? 0 : d > -63 ? -d : 63, r = d < 0 ? 0 : d < 63 ? d : 63;
-    return ((x << l) + (long long)((1ull << r) >> 1)) >> r;
+    return ((x << l) + (long long)(((1ull << r) - (unsigned)odd) >> 1)) >> r;
 }
 
 FXHD unsigned long long fx_dbits(double d)
